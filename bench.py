@@ -40,7 +40,7 @@ UNIT = "Gsample/s"
 # its own launch by the input samples the launch processes. Valid only for the
 # sources they were taken from (src = hash of the kernel's source files).
 KERNEL_SOURCES = {
-    "k_phase1": ['k_phase1.cuh', 'k_phase1_tile.inc', 'k_phase1_t1.cu', 'k_phase1_t2.cu', 'k_phase1_t4.cu', 'k_phase1_t8.cu', 'k_phase1_t16.cu', 'k_phase1_t32.cu', 'fe_device.cuh', 'fe_internal.cuh'],
+    "k_phase1": ['k_phase1.cuh', 'k_phase1_t1.cu', 'k_phase1_t2.cu', 'k_phase1_t4.cu', 'k_phase1_t8.cu', 'k_phase1_t16.cu', 'k_phase1_t32.cu', 'fe_device.cuh', 'fe_internal.cuh'],
     "k_phase2": ['k_phase2.cu', 'fe_device.cuh', 'fe_internal.cuh'],
     "k_phase2w": ['k_phase2w.cu', 'fe_device.cuh', 'fe_internal.cuh'],
     "k_phase1_tc": ['k_phase1_tc.cu', 'fe_device.cuh', 'fe_internal.cuh'],

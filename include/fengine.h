@@ -131,7 +131,7 @@ fengine_status fengine_default_weights(int32_t n_channels, int32_t n_taps, float
 
 /* The requantiser of one Gaussian-integer component that the kernels apply
  * (Sec. 2.1 step 6, Sec. 3.6): saturate to [-127, 127] and round half away
- * from zero, here evaluated on the host from the same source. */
+ * from zero, here evaluated on the host by the same steps. */
 int32_t fengine_quantise(float x);
 
 /* Create a plan on the current CUDA device (use the plan only while that

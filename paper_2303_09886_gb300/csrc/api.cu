@@ -704,7 +704,6 @@ fengine_status process_impl(fengine_plan_t pl, void *cuda_stream, const uint8_t 
     p1.ctab = pl->d_ctab;
     p1.window_tap = d_window_tap;
     p1.a_spectra = pl->SL;
-    p1.half_out = 0;
 
     fe::Phase2Params p2{};
     p2.tw2 = pl->d_tw2;
@@ -720,7 +719,8 @@ fengine_status process_impl(fengine_plan_t pl, void *cuda_stream, const uint8_t 
     p2.out = d_out;
     p2.prequant = reinterpret_cast<float2 *>(d_prequant);
     p2.a_spectra = pl->SL;
-    p2.half_in = pl->precision == FENGINE_TC_FP16;   // every form's second stage runs on CUDA cores
+    p2.in = pl->precision == FENGINE_TC_FP16 ? fe::kInHalf : pl->tc1 ? fe::kInFloat : fe::phase1_layout(pl->N1);
+    p2.err = pl->d_err;
     p2.tc_unscale = pl->tc_unscale;
 
     fe::Phase1TcParams pt{};
@@ -799,6 +799,7 @@ fengine_status process_impl(fengine_plan_t pl, void *cuda_stream, const uint8_t 
             p1.A = A;
             p1.q_begin = qb;
             p1.q_count = qc;
+            p1.rows = fe::phase1_rows(pl->T, pl->N1, pl->N2, qc, pl->n_streams);
             p2.A = A;
             p2.q_begin = qb;
             p2.q_count = qc;
@@ -858,6 +859,7 @@ fengine_status process_impl(fengine_plan_t pl, void *cuda_stream, const uint8_t 
         p1.A = A;
         p1.q_begin = qb;
         p1.q_count = qc;
+        p1.rows = fe::phase1_rows(pl->T, pl->N1, pl->N2, qc, pl->n_streams);
         pt.A = A;
         pt.q_begin = qb;
         pt.q_count = qc;

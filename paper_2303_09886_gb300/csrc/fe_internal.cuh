@@ -5,8 +5,8 @@
 //   k_phase1<T,N1>  unpack + coarse delay + PFB FIR (Eq. 1) + first FFT stage
 //                   (real N1-point DFT over t1, twiddle by exp(-2 pi i k1 t2 / N))
 //   k_phase2w       1024-point FFT over t2 + fine-delay rotation + gain +
-//                   requantise + channel-major corner turn (FP32 form,
-//                   persistent, one warp per sequence), or
+//                   requantise + channel-major corner turn (persistent, one
+//                   warp per pair of spectra), or
 //   k_phase2<N2>    the same for N2 < 1024
 // In the reduced-precision forms phase 1 is k_phase1_tc (tcgen05 tensor
 // cores: unpack + coarse delay + FIR + first DFT stage with its twiddle in one
@@ -85,17 +85,23 @@ struct Phase1Params {
     const float *w;           // [N*T] prototype, w[t + N j]
     const float2 *tw1;        // [(N1/2+1)][N2] exp(-2 pi i k1 t2 / N)
     const int *ctab;          // [stream][M]
-    float2 *A;                // out [stream][a_spectra][N1/2+1][N2], spectrum q at row q - q_begin
-                              // (FP16 pairs in 4-byte elements when half_out)
-    int half_out;             // 1: store B as FP16 (re, im) pairs (FP16 tensor-core form)
+    float2 *A;                // out, spectrum q at row q - q_begin: N1 <= 32 in spectrum pairs,
+                              // [stream][a_spectra / 2][N1/2+1][N2] of (re, re, im, im), else
+                              // [stream][a_spectra][N1/2+1][N2] of (re, im)
+    int rows;                 // spectra per CTA: even, at most kP1Blocks * kP1Block
     int *window_tap;          // optional out [stream][M][N]
     int q_begin, q_count;     // the slab of spectra this launch covers
     int a_spectra;            // spectra per stream in the intermediate buffer
 };
 
+// Layouts of the intermediate between the phases (a_spectra is even):
+constexpr int kInPairs = 0;   // FP32, [stream][a_spectra / 2][k1][t2] of (re, re, im, im) of two spectra
+constexpr int kInHalf = 1;    // FP16 (re, im) pairs, [stream][a_spectra][k1][t2] (tensor-core phase 1, FP16 form)
+constexpr int kInFloat = 2;   // FP32 (re, im), [stream][a_spectra][k1][t2] (BF16 form, and N1 = 64)
+inline int phase1_layout(int N1) { return N1 <= 32 ? kInPairs : kInFloat; }   // what k_phase1 writes
+
 struct Phase2Params {
-    const float2 *A;          // [stream][a_spectra][N1/2+1][N2], spectrum q at row q - q_begin
-                              // (FP16 pairs in 4-byte elements for the FP16 tensor-core form)
+    const float2 *A;          // the intermediate in the layout `in`, spectrum q at row q - q_begin
     int q_begin, q_count;     // the slab of spectra this launch covers
     int a_spectra;            // spectra per stream in the intermediate buffer
     const float2 *tw2;        // [N2] exp(-2 pi i q / N2)
@@ -106,7 +112,8 @@ struct Phase2Params {
     int N, N1, M, S, R2;      // FFT length, first-stage size, spectra/call, spectra/heap, spectra/CTA
     int8_t *out;              // [ant][heap][n][S_h][pol][2]
     float2 *prequant;         // optional [stream][M][n]
-    int half_in;              // 1: A holds FP16 (re, im) pairs (tensor-core phase 1, FP16 form)
+    int in;                   // layout of A: kInPairs, kInHalf or kInFloat
+    int *err;                 // set to 2 if a bounded wait gave up (may be nullptr)
     float tc_unscale;         // inverse of the power-of-two scale of an FP16 A (1 otherwise)
 };
 
@@ -117,35 +124,34 @@ cudaError_t launch_tail_update(const uint8_t *hist_in, const uint8_t *chunk, uin
                                cudaStream_t s);
 cudaError_t launch_phase1(int T, int N1, const Phase1Params &p, int n_streams, cudaStream_t s);
 cudaError_t launch_phase2(int N2, const Phase2Params &p, int n_ant, cudaStream_t s);
-// FP32 second stage for N2 = 1024 (launch_phase2 routes it there): one warp
-// per sequence, two in-register 32-point DFTs around one shared-memory transpose
-cudaError_t launch_phase2w(const Phase2Params &p, int n_ant, cudaStream_t s);
-size_t phase2w_smem_bytes();
 
 // ---- grouped launches (batching): the launches of several plans that use
 // one kernel instantiation, as one grid. Member m owns the blocks
 // [start[m], start[m + 1]) and runs with parameters p[m]. The whole group is
 // passed by value as the kernel's parameter (at most kMaxGroup members, a
 // few KB), so a grouped launch is captured into a CUDA graph like any other.
+// A single plan's launch is a group of one member (CAP = 1).
 constexpr int kMaxGroup = 64;
-template <class P>
+template <class P, int CAP>
 struct GroupArgs {
-    P p[kMaxGroup];
-    int start[kMaxGroup + 1];   // start[n] = blocks of the launch
-    int aux[kMaxGroup];         // the member's blocks along y (grid kernels) or antennas (k_phase2w)
+    P p[CAP];
+    int start[CAP + 1];         // start[n] = blocks of the launch
+    int aux[CAP];               // the member's blocks along y (grid kernels) or antennas (k_phase2w)
     int gx;                     // blocks along x, the same for every member (grid kernels)
     int n;
 };
-using Phase1Group = GroupArgs<Phase1Params>;
-using Phase2Group = GroupArgs<Phase2Params>;
+using Phase1Group = GroupArgs<Phase1Params, kMaxGroup>;
+using Phase2Group = GroupArgs<Phase2Params, kMaxGroup>;
 // one member's blocks and their (gx, gy) in its own launch
 int phase1_blocks(int N1, const Phase1Params &p, int n_streams, int *gx, int *gy);
 int phase2_blocks(int N2, const Phase2Params &p, int n_ant, int *gx, int *gy);   // N2 < 1024
 long long phase2w_items(const Phase2Params &p, int n_ant);                        // work items of k_phase2w
 int phase2w_wave();                                                                 // CTAs of one k_phase2w wave
 cudaError_t launch_phase1_group(int T, int N1, const Phase1Group &g, cudaStream_t s);
-cudaError_t launch_phase2_group(int N2, bool half_in, const Phase2Group &g, cudaStream_t s);
-cudaError_t launch_phase2w_group(bool half_in, const Phase2Group &g, cudaStream_t s);
+cudaError_t launch_phase2_group(int N2, int in, const Phase2Group &g, cudaStream_t s);
+// second stage for N2 = 1024 (launch_phase2 and launch_phase2_group route it there)
+cudaError_t launch_phase2w(const Phase2Params &p, int n_ant, cudaStream_t s);
+cudaError_t launch_phase2w_group(int in, const Phase2Group &g, cudaStream_t s);
 
 // A call of a plan with its phase launches handed back instead of enqueued
 // (batching): the per-slab parameters fengine_process_chunk would launch.
@@ -167,7 +173,9 @@ fengine_status process_chunk_deferred(fengine_plan_t pl, cudaStream_t st, const 
                                       bool *deferred);
 
 // Tile shapes (host and device agree through these).
-constexpr int kP1Rows = 32;   // spectra per phase-1 CTA
+constexpr int kP1Block = 32;   // spectra per block of a phase-1 tile (one DFT stage)
+constexpr int kP1Blocks = 4;   // blocks per phase-1 tile at most
+int phase1_rows(int T, int N1, int N2, int q_count, int n_streams);   // spectra per phase-1 CTA
 inline int phase1_W(int N1, int N2) {
     int w = 512 / N1;           // 512 FIR columns per tile
     return w < N2 ? w : N2;

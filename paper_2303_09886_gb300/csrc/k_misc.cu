@@ -5,42 +5,65 @@
 
 namespace fe {
 
-template <int T>
-cudaError_t launch_phase1_n1(int N1, const Phase1Params &p, int n_streams, cudaStream_t s);
-template <int T>
-cudaError_t launch_phase1_group_n1(int N1, const Phase1Group &g, cudaStream_t s);
+template <int T, int CAP>
+cudaError_t launch_phase1_n1(int N1, const GroupArgs<Phase1Params, CAP> &g, cudaStream_t s);
 
-cudaError_t launch_phase1_group(int T, int N1, const Phase1Group &g, cudaStream_t s) {
+template <int CAP>
+static cudaError_t launch_phase1_t(int T, int N1, const GroupArgs<Phase1Params, CAP> &g, cudaStream_t s) {
     switch (T) {
-        case 1: return launch_phase1_group_n1<1>(N1, g, s);
-        case 2: return launch_phase1_group_n1<2>(N1, g, s);
-        case 4: return launch_phase1_group_n1<4>(N1, g, s);
-        case 8: return launch_phase1_group_n1<8>(N1, g, s);
-        case 16: return launch_phase1_group_n1<16>(N1, g, s);
-        case 32: return launch_phase1_group_n1<32>(N1, g, s);
+        case 1: return launch_phase1_n1<1, CAP>(N1, g, s);
+        case 2: return launch_phase1_n1<2, CAP>(N1, g, s);
+        case 4: return launch_phase1_n1<4, CAP>(N1, g, s);
+        case 8: return launch_phase1_n1<8, CAP>(N1, g, s);
+        case 16: return launch_phase1_n1<16, CAP>(N1, g, s);
+        case 32: return launch_phase1_n1<32, CAP>(N1, g, s);
         default: return cudaErrorInvalidValue;
     }
 }
 
-// the grid launch_phase1 uses: (N2 / W, tiles of kP1Rows spectra, streams)
+cudaError_t launch_phase1_group(int T, int N1, const Phase1Group &g, cudaStream_t s) {
+    return launch_phase1_t<kMaxGroup>(T, N1, g, s);
+}
+
+// blocks of a launch: (t2 blocks, tiles of p.rows spectra, streams)
 int phase1_blocks(int N1, const Phase1Params &p, int n_streams, int *gx, int *gy) {
     (void)N1;
     *gx = p.N2 / p.W;
-    *gy = (p.q_count + kP1Rows - 1) / kP1Rows;
+    *gy = (p.q_count + p.rows - 1) / p.rows;
     return *gx * *gy * n_streams;
 }
 
-
 cudaError_t launch_phase1(int T, int N1, const Phase1Params &p, int n_streams, cudaStream_t s) {
-    switch (T) {
-        case 1: return launch_phase1_n1<1>(N1, p, n_streams, s);
-        case 2: return launch_phase1_n1<2>(N1, p, n_streams, s);
-        case 4: return launch_phase1_n1<4>(N1, p, n_streams, s);
-        case 8: return launch_phase1_n1<8>(N1, p, n_streams, s);
-        case 16: return launch_phase1_n1<16>(N1, p, n_streams, s);
-        case 32: return launch_phase1_n1<32>(N1, p, n_streams, s);
-        default: return cudaErrorInvalidValue;
+    GroupArgs<Phase1Params, 1> g;
+    g.p[0] = p;
+    g.start[0] = 0;
+    g.start[1] = phase1_blocks(N1, p, n_streams, &g.gx, &g.aux[0]);
+    g.n = 1;
+    return launch_phase1_t<1>(T, N1, g, s);
+}
+
+// Spectra per phase-1 CTA. More rows share the T - 1 lead-in rows, the weights
+// and the twiddles; fewer give more CTAs. Costs in rows: a filtered row 1, a
+// lead-in row about 0.3 of it, a CTA's start-up and DFT latency about 8; the
+// launch takes ceil(CTAs / resident CTAs) rounds of that.
+int phase1_rows(int T, int N1, int N2, int q_count, int n_streams) {
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
+        sms = 148;
+    const long long slots = 2LL * sms, cols = (long long)(N2 / phase1_W(N1, N2)) * n_streams;
+    int best = kP1Block;
+    double best_cost = -1.0;
+    for (int rows : {128, 64, 32, 16, 8}) {
+        const long long ctas = cols * ((q_count + rows - 1) / rows);
+        const int used = rows < q_count ? rows : q_count;
+        const double cost = (double)((ctas + slots - 1) / slots) * (used + 0.3 * (T - 1) + 8.0);
+        if (best_cost < 0.0 || cost < best_cost) {
+            best = rows;
+            best_cost = cost;
+        }
     }
+    return best;
 }
 
 // Delay model per spectrum (Sec. 2.1 steps 2 and 4, Sec. 3.3): for the

@@ -156,8 +156,13 @@ __device__ __forceinline__ int dif_pos(int k2) {
 
 }  // namespace
 
-template <int N2, bool HALF_IN>
-__global__ void __launch_bounds__(kP2Threads, 3) k_phase2(const Phase2Params p) {
+// The tiles of one plan's second stage (CAP = 1) or of several plans' (same
+// N2) in one grid.
+template <int N2, int IN, int CAP>
+__global__ void __launch_bounds__(kP2Threads, 3) k_phase2(const __grid_constant__ GroupArgs<Phase2Params, CAP> ga) {
+    const int m = CAP == 1 ? 0 : group_member(ga, (int)blockIdx.x);
+    const Phase2Params &p = ga.p[m];
+    const int blk = (int)blockIdx.x - (CAP == 1 ? 0 : ga.start[m]), gy = ga.aux[m];
     using S = P2Shape<N2>;
     constexpr int R2 = S::R2, LD = S::LD;
     extern __shared__ float2 sm[];
@@ -169,39 +174,8 @@ __global__ void __launch_bounds__(kP2Threads, 3) k_phase2(const Phase2Params p) 
     long long *rowoff = reinterpret_cast<long long *>(qup + 2 * R2);   // [R2] heap row byte offset
     int *rowstride = reinterpret_cast<int *>(rowoff + R2);             // [R2] bytes per channel row
 
-    const int k1 = blockIdx.x, ant = blockIdx.z;
-    const int q0 = p.q_begin + blockIdx.y * R2;
-#include "k_phase2_tile.inc"
-}
-
-// The tiles of several plans' second stages (same N2) in one grid.
-template <int N2, bool HALF_IN>
-__global__ void __launch_bounds__(kP2Threads, 3) k_phase2_group(const Phase2Group g) {
-    __shared__ Phase2Params sp;
-    __shared__ int sxyz[3];
-    if (threadIdx.x == 0) {
-        const int m = group_member(g, (int)blockIdx.x);
-        const int b = (int)blockIdx.x - g.start[m], gy = g.aux[m];
-        sxyz[0] = b % g.gx;
-        sxyz[1] = (b / g.gx) % gy;
-        sxyz[2] = b / (g.gx * gy);
-        sp = g.p[m];
-    }
-    __syncthreads();
-    const Phase2Params &p = sp;
-    using S = P2Shape<N2>;
-    constexpr int R2 = S::R2, LD = S::LD;
-    extern __shared__ float2 sm[];
-    float2 *buf = sm;                                  // [2 R2][LD]
-    constexpr int HP = S::HI + 1, LP = S::LO + 1;      // padded table rows (no bank conflicts)
-    float2 *thi = buf + 2 * R2 * LD;                   // [2 R2][HP]
-    float2 *tlo = thi + 2 * R2 * HP;                   // [2 R2][LP]
-    float2 *qup = tlo + 2 * R2 * LP;                   // [2 R2] upper-class factor
-    long long *rowoff = reinterpret_cast<long long *>(qup + 2 * R2);   // [R2] heap row byte offset
-    int *rowstride = reinterpret_cast<int *>(rowoff + R2);             // [R2] bytes per channel row
-
-    const int k1 = sxyz[0], ant = sxyz[2];
-    const int q0 = p.q_begin + sxyz[1] * R2;
+    const int k1 = blk % ga.gx, ant = blk / (ga.gx * gy);
+    const int q0 = p.q_begin + ((blk / ga.gx) % gy) * R2;
 #include "k_phase2_tile.inc"
 }
 
@@ -212,25 +186,7 @@ size_t phase2_smem_bytes(int N2, int R2) {
            (sizeof(long long) + sizeof(int)) * R2;
 }
 
-template <int N2, bool HALF_IN>
-static cudaError_t launch_p2h(const Phase2Params &p, int n_ant, cudaStream_t s) {
-    const int R2 = P2Shape<N2>::R2;
-    if (p.R2 != R2) return cudaErrorInvalidValue;
-    const size_t smem = phase2_smem_bytes(N2, R2);
-    cudaError_t e = cudaFuncSetAttribute(k_phase2<N2, HALF_IN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
-    if (e != cudaSuccess) return e;
-    dim3 grid(p.N1 / 2 + 1, (p.q_count + R2 - 1) / R2, n_ant);
-    k_phase2<N2, HALF_IN><<<grid, kP2Threads, smem, s>>>(p);
-    return cudaGetLastError();
-}
-
-template <int N2>
-static cudaError_t launch_p2(const Phase2Params &p, int n_ant, cudaStream_t s) {
-    return p.half_in ? launch_p2h<N2, true>(p, n_ant, s) : launch_p2h<N2, false>(p, n_ant, s);
-}
-
-// the grid launch_phase2 uses for N2 < 1024: (classes k1, tiles of R2 spectra, antennas)
+// the grid for N2 < 1024: (classes k1, tiles of R2 spectra, antennas)
 int phase2_blocks(int N2, const Phase2Params &p, int n_ant, int *gx, int *gy) {
     (void)N2;
     *gx = p.N1 / 2 + 1;
@@ -238,55 +194,57 @@ int phase2_blocks(int N2, const Phase2Params &p, int n_ant, int *gx, int *gy) {
     return *gx * *gy * n_ant;
 }
 
-template <int N2, bool HALF_IN>
-static cudaError_t launch_p2h_group(const Phase2Group &g, cudaStream_t s) {
+template <int N2, int IN, int CAP>
+static cudaError_t launch_p2(const GroupArgs<Phase2Params, CAP> &g, cudaStream_t s) {
     const int R2 = P2Shape<N2>::R2;
     const size_t smem = phase2_smem_bytes(N2, R2);
-    cudaError_t e = cudaFuncSetAttribute(k_phase2_group<N2, HALF_IN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
+    cudaError_t e =
+        cudaFuncSetAttribute(k_phase2<N2, IN, CAP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     for (int m = 0; m < g.n; m++)
-        if (g.p[m].R2 != R2) return cudaErrorInvalidValue;
+        if (g.p[m].R2 != R2 || g.p[m].a_spectra % 2) return cudaErrorInvalidValue;
     if (g.n < 1 || g.start[g.n] < 1) return cudaSuccess;
-    k_phase2_group<N2, HALF_IN><<<g.start[g.n], kP2Threads, smem, s>>>(g);
+    k_phase2<N2, IN, CAP><<<g.start[g.n], kP2Threads, smem, s>>>(g);
     return cudaGetLastError();
 }
 
-template <int N2>
-static cudaError_t launch_p2_group(bool half_in, const Phase2Group &g, cudaStream_t s) {
-    return half_in ? launch_p2h_group<N2, true>(g, s) : launch_p2h_group<N2, false>(g, s);
+template <int N2, int CAP>
+static cudaError_t launch_p2_in(int in, const GroupArgs<Phase2Params, CAP> &g, cudaStream_t s) {
+    switch (in) {
+        case kInPairs: return launch_p2<N2, kInPairs, CAP>(g, s);
+        case kInHalf: return launch_p2<N2, kInHalf, CAP>(g, s);
+        default: return launch_p2<N2, kInFloat, CAP>(g, s);
+    }
 }
 
-cudaError_t launch_phase2_group(int N2, bool half_in, const Phase2Group &g, cudaStream_t s) {
+template <int CAP>
+static cudaError_t launch_p2_n2(int N2, int in, const GroupArgs<Phase2Params, CAP> &g, cudaStream_t s) {
     switch (N2) {
-        case 2: return launch_p2_group<2>(half_in, g, s);
-        case 4: return launch_p2_group<4>(half_in, g, s);
-        case 8: return launch_p2_group<8>(half_in, g, s);
-        case 16: return launch_p2_group<16>(half_in, g, s);
-        case 32: return launch_p2_group<32>(half_in, g, s);
-        case 64: return launch_p2_group<64>(half_in, g, s);
-        case 128: return launch_p2_group<128>(half_in, g, s);
-        case 256: return launch_p2_group<256>(half_in, g, s);
-        case 512: return launch_p2_group<512>(half_in, g, s);
-        case 1024: return launch_phase2w_group(half_in, g, s);
+        case 2: return launch_p2_in<2>(in, g, s);
+        case 4: return launch_p2_in<4>(in, g, s);
+        case 8: return launch_p2_in<8>(in, g, s);
+        case 16: return launch_p2_in<16>(in, g, s);
+        case 32: return launch_p2_in<32>(in, g, s);
+        case 64: return launch_p2_in<64>(in, g, s);
+        case 128: return launch_p2_in<128>(in, g, s);
+        case 256: return launch_p2_in<256>(in, g, s);
+        case 512: return launch_p2_in<512>(in, g, s);
         default: return cudaErrorInvalidValue;
     }
+}
+
+cudaError_t launch_phase2_group(int N2, int in, const Phase2Group &g, cudaStream_t s) {
+    return N2 == 1024 ? launch_phase2w_group(in, g, s) : launch_p2_n2(N2, in, g, s);
 }
 
 cudaError_t launch_phase2(int N2, const Phase2Params &p, int n_ant, cudaStream_t s) {
-    switch (N2) {
-        case 2: return launch_p2<2>(p, n_ant, s);
-        case 4: return launch_p2<4>(p, n_ant, s);
-        case 8: return launch_p2<8>(p, n_ant, s);
-        case 16: return launch_p2<16>(p, n_ant, s);
-        case 32: return launch_p2<32>(p, n_ant, s);
-        case 64: return launch_p2<64>(p, n_ant, s);
-        case 128: return launch_p2<128>(p, n_ant, s);
-        case 256: return launch_p2<256>(p, n_ant, s);
-        case 512: return launch_p2<512>(p, n_ant, s);
-        case 1024: return launch_phase2w(p, n_ant, s);   // one warp per 1024-point sequence
-        default: return cudaErrorInvalidValue;
-    }
+    if (N2 == 1024) return launch_phase2w(p, n_ant, s);   // one warp per pair of 1024-point sequences
+    GroupArgs<Phase2Params, 1> g;
+    g.p[0] = p;
+    g.start[0] = 0;
+    g.start[1] = phase2_blocks(N2, p, n_ant, &g.gx, &g.aux[0]);
+    g.n = 1;
+    return launch_p2_n2(N2, p.in, g, s);
 }
 
 }  // namespace fe

@@ -226,6 +226,7 @@ fengine_status fengine_process_chunk_noalloc(const fengine_noalloc_args *a, cons
     p2.R2 = fe::phase2_R2(N2);
     p2.out = d_out;
     p2.prequant = nullptr;
+    p2.in = fe::phase1_layout(N1);
     p2.a_spectra = (int)SL;
 
     // one intermediate buffer: slabs run back to back on the caller's stream
@@ -233,6 +234,7 @@ fengine_status fengine_process_chunk_noalloc(const fengine_noalloc_args *a, cons
         const int qc = (int)((M - qb) < SL ? (M - qb) : SL);
         p1.q_begin = p2.q_begin = (int)qb;
         p1.q_count = p2.q_count = qc;
+        p1.rows = fe::phase1_rows(T, N1, N2, qc, ns);
         if (fe::launch_phase1(T, N1, p1, ns, st) != cudaSuccess) return FENGINE_ECUDA;
         if (fe::launch_phase2(N2, p2, nant, st) != cudaSuccess) return FENGINE_ECUDA;
     }
