@@ -242,9 +242,8 @@ def _base_streams(seed: int, n: int, sigma: float = 32.0):
 
 
 def _batched_launches(plans):
-    """Kernel launches of one fengine_batch_process over FP32 plans: a delay
-    table and a history-tail update per member (and the lost-data flags when
-    its chunks are heap-aligned), then per group of members with the same
+    """Kernel launches of one fengine_batch_process over FP32 plans: one for
+    the delay table, lost-data flags and history tail per member, then per group of members with the same
     (taps, N1, N2), one phase-1 and one phase-2 grid per slab round (at most
     64 members per grid)."""
     groups = {}
@@ -255,8 +254,7 @@ def _batched_launches(plans):
         for r in range(max(slabs)):
             k = sum(1 for s in slabs if s > r)
             grids += 2 * ((k + 63) // 64)
-    small = sum(2 + (1 if p.chunk_samples % 4096 == 0 else 0) for p in plans)
-    return small + grids
+    return len(plans) + grids
 
 
 def run_batched(args):
@@ -523,9 +521,9 @@ def run_narrowband(args, wl):
             "warmup": 3, "ms_per_step": r["ddc_and_plan"]["ms_per_step"], "higher_is_better": True,
             "scaling": "weak", "vs_baseline": None, "dtype": "f32", "data": "synthetic",
             "config": {"workload": "narrow-band mode on " + wl.description, **r["config"]},
-            # per step: the down-converter and its history tail, then the plan's delay table,
-            # lost-data flags, phase 1, phase 2 and history tail
-            "ddc_only": r["ddc_only"], "gpu_launches": 7 * max(3, min(args.steps, 20))}
+            # per step: the down-converter and its history tail, then the plan's first kernel
+            # (delay table, lost-data flags, history tail), phase 1 and phase 2
+            "ddc_only": r["ddc_only"], "gpu_launches": 5 * max(3, min(args.steps, 20))}
     print(json.dumps(line), flush=True)
     return 0
 
@@ -836,10 +834,9 @@ def main(argv=None):
                  "with_intermediates_GBps": path_all, "frac_with_intermediates": path_all / peak,
                  "bytes_per_sample": {"algorithmic": 2.25, "with_intermediates": 2.25 + 2 * inter}},
         "e2e": e2e,
-        # delay table, history tail, lost-data flags (heap-aligned chunks),
-        # the column unpack (tensor-core forms), a phase-1 / phase-2 pair per slab
-        "gpu_launches": (2 + (1 if wl.chunk_samples % 4096 == 0 else 0) + (1 if tc else 0) + 2 * slabs)
-        * args.steps,
+        # one for the delay table, lost-data flags and history tail, the column
+        # unpack (tensor-core forms), a phase-1 / phase-2 pair per slab
+        "gpu_launches": (1 + (1 if tc else 0) + 2 * slabs) * args.steps,
         "forms": forms,
         "clocks": clocks.summary(w0, w1),
         **extra,

@@ -94,7 +94,8 @@ typedef struct {
                                   with N2 <= 1024 (and N2 >= 512 / N1 for N1 > 8);
                                   built-in: max(8, N / 1024) */
     int32_t slab_spectra;      /* spectra per slab of the two-phase pipeline, a multiple
-                                  of 32; built-in: an FP32 intermediate of about 256 MiB */
+                                  of 32; built-in: an intermediate of about 3 GiB (less
+                                  where the device has no room for it) */
     int64_t min_delay_samples; /* Dmin in [-2^30, 0]: the most negative coarse delay
                                   (Sec. 3.3 allows negative delays). The plan emits
                                   E = ceil(-Dmin / 2n) spectra later to make room. */

@@ -319,22 +319,46 @@ fengine_status fengine_plan_create(const fengine_config *cfg, fengine_plan_t *ou
 
     const int ns = pl->n_streams;
     cudaError_t e = cudaSuccess;
+    if ((!tc1 && (e = fe::prepare_phase1(T, N1, pl->W)) != cudaSuccess) ||
+        (e = fe::prepare_phase2(pl->N2, tc1 ? (cfg->precision == FENGINE_TC_FP16 ? fe::kInHalf : fe::kInFloat)
+                                            : fe::phase1_layout(N1))) != cudaSuccess) {
+        release(pl);
+        return cuda_fail(e, "kernel attributes");
+    }
     // Slab of spectra per phase-1 / phase-2 launch pair: built-in, the
-    // spectra whose FP32 intermediate (all streams) is about 256 MiB, a
-    // multiple of 32 (both phases' tiles). Measured on GB300 (fengine_autotune),
-    // launches over more spectra win over keeping a smaller intermediate in
-    // L2: the grids then span several waves of CTAs.
+    // spectra whose intermediate (all streams) is about 3 GiB, a multiple of
+    // 32 (both phases' tiles): the whole chunk of every workload here, in one
+    // buffer and one launch pair. Neither phase is bound by memory (the second
+    // stage takes the same time per spectrum from L2), so smaller slabs only
+    // add launches and tails: 8192 channels, 4 antennas x 2 x 2^25 samples
+    // take 0.89 ms as one slab and 1.02 ms as five of 256 MiB. Where the
+    // device has no room for it, down to the 256 MiB slab.
     // intermediate element: FP32 (re, im), or FP16 (re, im) in the FP16 form
     pl->a_elem = pl->precision == FENGINE_TC_FP16 ? 4 : 8;
     const size_t per_spec = (size_t)ns * (pl->N1 / 2 + 1) * pl->N2 * pl->a_elem;
-    long long SL = cfg->slab_spectra ? cfg->slab_spectra : (long long)((256u << 20) / per_spec) / 32 * 32;
-    if (SL < 32) SL = 32;
     const long long M32 = (M + 31) / 32 * 32;
-    if (SL > M32) SL = M32;
+    auto slab_of = [&](size_t bytes) {
+        long long s = (long long)(bytes / per_spec) / 32 * 32;
+        if (s < 32) s = 32;
+        return s > M32 ? M32 : s;
+    };
+    const long long SL_min = slab_of((size_t)256 << 20);
+    long long SL = cfg->slab_spectra ? (cfg->slab_spectra > M32 ? M32 : cfg->slab_spectra) : slab_of((size_t)3 << 30);
+    size_t a_bytes = 0;
+    for (;;) {
+        a_bytes = (size_t)((M + SL - 1) / SL > 1 ? 2 : 1) * SL * per_spec;
+        e = dalloc(pl, &pl->d_A, a_bytes);
+        if (e == cudaSuccess || cfg->slab_spectra || SL <= SL_min) break;
+        cudaGetLastError();
+        SL = SL / 64 * 32 > SL_min ? SL / 64 * 32 : SL_min;
+    }
+    if (e != cudaSuccess) {
+        release(pl);
+        g_last_error = std::string("device allocation: ") + cudaGetErrorString(e);
+        return FENGINE_ENOMEM;
+    }
     pl->SL = (int)SL;
     pl->n_slabs = (int)((M + SL - 1) / SL);
-    const int nbuf = pl->n_slabs > 1 ? 2 : 1;
-    const size_t a_bytes = (size_t)nbuf * SL * per_spec;
     if ((e = dalloc(pl, &pl->d_w, sizeof(float) * N * T)) != cudaSuccess ||
         (e = dalloc(pl, &pl->d_tw1, sizeof(float2) * (pl->N1 / 2 + 1) * pl->N2)) != cudaSuccess ||
         (e = dalloc(pl, &pl->d_tw2, sizeof(float2) * pl->N2)) != cudaSuccess ||
@@ -347,7 +371,6 @@ fengine_status fengine_plan_create(const fengine_config *cfg, fengine_plan_t *ou
         (e = dalloc(pl, &pl->d_hvalid[1], (size_t)ns * pl->HV)) != cudaSuccess ||
         (e = dalloc(pl, &pl->d_ftab, sizeof(float2) * ns * M)) != cudaSuccess ||
         (e = dalloc(pl, &pl->d_ctab, sizeof(int) * ns * M)) != cudaSuccess ||
-        (e = dalloc(pl, &pl->d_A, a_bytes)) != cudaSuccess ||
         (e = dalloc(pl, &pl->d_hist[0], (size_t)pl->hist_bytes * ns + 16)) != cudaSuccess ||
         (e = dalloc(pl, &pl->d_hist[1], (size_t)pl->hist_bytes * ns + 16)) != cudaSuccess ||
         (e = dalloc(pl, &pl->d_seg, sizeof(DelaySeg) * fe::kMaxSeg * ns)) != cudaSuccess ||
@@ -657,22 +680,20 @@ fengine_status process_impl(fengine_plan_t pl, void *cuda_stream, const uint8_t 
     dp.g_tapply = pl->d_gtap;
     dp.n_gsets = pl->d_ngs;
     dp.gsel = pl->d_gsel;
-    dp.cchg = pl->d_cchg;
-    prof_begin(pl, 0, st);
-    if ((e = fe::launch_delay_table(dp, st)) != cudaSuccess) return cuda_fail(e, "delay table launch");
-    prof_end(pl, st);
-
+    dp.cchg = pl->tc1 ? pl->d_cchg : nullptr;   // only the tensor-core phase 1 reads it
     // Lost data (Sec. 3.7): heap flags of this call and the history heaps'
     // received flags for the next one (kept whenever the call is heap-aligned)
+    fe::PrologueParams pp{};
+    pp.d = dp;
     if (heap_aligned) {
-        fe::LostDataParams lp{};
+        fe::LostDataParams &lp = pp.l;
+        pp.lost = 1;
         lp.valid = d_valid;
         lp.hv_in = pl->d_hvalid[pl->cur];
         lp.hv_out = pl->d_hvalid[1 - pl->cur];
         lp.HV = pl->HV;
         lp.heap0 = first_sample / fe::kHeapSamples;
         lp.chunk_heaps = (int)(pl->L / fe::kHeapSamples);
-        lp.ctab = pl->d_ctab;
         lp.n_ant = pl->n_ant;
         lp.N = pl->N;
         lp.T = pl->T;
@@ -680,10 +701,19 @@ fengine_status process_impl(fengine_plan_t pl, void *cuda_stream, const uint8_t 
         lp.S = pl->S;
         lp.m0 = m0;
         lp.heap_flags = d_heap_flags;
-        if ((e = fe::launch_lost_data(lp, st)) != cudaSuccess) return cuda_fail(e, "lost-data launch");
     } else if (pl->lost_ok) {
         pl->hv_known = false;
     }
+    // the history for the next call (the buffer this call does not read)
+    pp.hist_in = pl->d_hist[pl->cur];
+    pp.chunk = d_packed;
+    pp.hist_out = pl->d_hist[1 - pl->cur];
+    pp.tail_bytes = pl->hist_bytes;
+    pp.chunk_bytes = pl->chunk_bytes;
+    pp.n_streams = pl->n_streams;
+    prof_begin(pl, 0, st);
+    if ((e = fe::launch_prologue(pp, st)) != cudaSuccess) return cuda_fail(e, "prologue launch");
+    prof_end(pl, st);
 
     fe::Phase1Params p1{};
     p1.chunk = d_packed;
@@ -757,7 +787,7 @@ fengine_status process_impl(fengine_plan_t pl, void *cuda_stream, const uint8_t 
         up.plane_elems = (long long)pl->n_streams * (pl->N / 8) * pl->cols_rtp;
         if (!split_unpack) {
             prof_begin(pl, 4, st);
-            if ((e = fe::launch_unpack_cols(up, st)) != cudaSuccess) return cuda_fail(e, "unpack launch");
+            if ((e = fe::launch_unpack_cols(up, st, true)) != cudaSuccess) return cuda_fail(e, "unpack launch");
             prof_end(pl, st);
         }
         pt.cols = pl->d_cols;
@@ -781,9 +811,6 @@ fengine_status process_impl(fengine_plan_t pl, void *cuda_stream, const uint8_t 
 
     if (def) {
         const size_t slab_elems = (size_t)pl->n_streams * pl->SL * (pl->N1 / 2 + 1) * pl->N2;
-        if ((e = fe::launch_tail_update(pl->d_hist[pl->cur], d_packed, pl->d_hist[1 - pl->cur], pl->hist_bytes,
-                                        pl->chunk_bytes, pl->n_streams, st)) != cudaSuccess)
-            return cuda_fail(e, "tail launch");
         def->T = pl->T;
         def->N1 = pl->N1;
         def->N2 = pl->N2;
@@ -816,12 +843,16 @@ fengine_status process_impl(fengine_plan_t pl, void *cuda_stream, const uint8_t 
     // Slab pipeline: slab s uses intermediate buffer s % 2; phase 1 runs on
     // internal stream 0, phase 2 on internal stream 1, so phase 1 of slab
     // s + 1 overlaps phase 2 of slab s. Buffer reuse waits for phase 2 of
-    // slab s - 2. Both internal streams fork from and join back into st.
+    // slab s - 2. Both internal streams fork from and join back into st. A
+    // call of one slab has nothing to overlap: its kernels follow each other
+    // on st itself, each beginning under the end of the one before.
     const size_t slab_elems = (size_t)pl->n_streams * pl->SL * (pl->N1 / 2 + 1) * pl->N2;
-    if ((e = cudaEventRecord(pl->ev_fork, st)) != cudaSuccess ||
-        (e = cudaStreamWaitEvent(pl->sp[0], pl->ev_fork, 0)) != cudaSuccess ||
-        (e = cudaStreamWaitEvent(pl->sp[1], pl->ev_fork, 0)) != cudaSuccess ||
-        (split_unpack && (e = cudaStreamWaitEvent(pl->sp[2], pl->ev_fork, 0)) != cudaSuccess))
+    const bool one = pl->n_slabs == 1;
+    const cudaStream_t s1 = one ? st : pl->sp[0], s2 = one ? st : pl->sp[1];
+    if (!one && ((e = cudaEventRecord(pl->ev_fork, st)) != cudaSuccess ||
+                 (e = cudaStreamWaitEvent(s1, pl->ev_fork, 0)) != cudaSuccess ||
+                 (e = cudaStreamWaitEvent(s2, pl->ev_fork, 0)) != cudaSuccess ||
+                 (split_unpack && (e = cudaStreamWaitEvent(pl->sp[2], pl->ev_fork, 0)) != cudaSuccess)))
         return cuda_fail(e, "slab fork");
     int unpacked = 0;   // column rows [0, unpacked) enqueued so far
     for (int s = 0; s < pl->n_slabs; s++) {
@@ -829,7 +860,7 @@ fengine_status process_impl(fengine_plan_t pl, void *cuda_stream, const uint8_t 
         float2 *A = reinterpret_cast<float2 *>(reinterpret_cast<char *>(pl->d_A) + (size_t)b * slab_elems * pl->a_elem);
         const int qb = s * pl->SL;
         const int qc = (pl->M - qb) < pl->SL ? (pl->M - qb) : pl->SL;
-        if (s >= 2 && (e = cudaStreamWaitEvent(pl->sp[0], pl->ev_p2[b], 0)) != cudaSuccess)
+        if (s >= 2 && (e = cudaStreamWaitEvent(s1, pl->ev_p2[b], 0)) != cudaSuccess)
             return cuda_fail(e, "slab wait");
         if (split_unpack) {
             // the rows this slab's passes can read: the last tile's column
@@ -848,12 +879,12 @@ fengine_status process_impl(fengine_plan_t pl, void *cuda_stream, const uint8_t 
                 up.row_begin = unpacked;
                 up.row_end = hi;
                 prof_begin(pl, 4, pl->sp[2]);
-                if ((e = fe::launch_unpack_cols(up, pl->sp[2])) != cudaSuccess) return cuda_fail(e, "unpack launch");
+                if ((e = fe::launch_unpack_cols(up, pl->sp[2], false)) != cudaSuccess) return cuda_fail(e, "unpack launch");
                 prof_end(pl, pl->sp[2]);
                 unpacked = hi;
             }
             if ((e = cudaEventRecord(pl->ev_u[b], pl->sp[2])) != cudaSuccess ||
-                (e = cudaStreamWaitEvent(pl->sp[0], pl->ev_u[b], 0)) != cudaSuccess)
+                (e = cudaStreamWaitEvent(s1, pl->ev_u[b], 0)) != cudaSuccess)
                 return cuda_fail(e, "unpack handoff");
         }
         p1.A = A;
@@ -863,33 +894,28 @@ fengine_status process_impl(fengine_plan_t pl, void *cuda_stream, const uint8_t 
         pt.A = A;
         pt.q_begin = qb;
         pt.q_count = qc;
-        prof_begin(pl, 1, pl->sp[0]);
-        if ((e = pl->tc1 ? fe::launch_phase1_tc(pl->T, pl->precision, pt, pl->sp[0])
-                         : fe::launch_phase1(pl->T, pl->N1, p1, pl->n_streams, pl->sp[0])) != cudaSuccess)
+        prof_begin(pl, 1, s1);
+        if ((e = pl->tc1 ? fe::launch_phase1_tc(pl->T, pl->precision, pt, s1, one)
+                         : fe::launch_phase1(pl->T, pl->N1, p1, pl->n_streams, s1, one)) != cudaSuccess)
             return cuda_fail(e, "phase-1 launch");
-        prof_end(pl, pl->sp[0]);
-        if ((e = cudaEventRecord(pl->ev_p1[b], pl->sp[0])) != cudaSuccess ||
-            (e = cudaStreamWaitEvent(pl->sp[1], pl->ev_p1[b], 0)) != cudaSuccess)
+        prof_end(pl, s1);
+        if (!one && ((e = cudaEventRecord(pl->ev_p1[b], s1)) != cudaSuccess ||
+                     (e = cudaStreamWaitEvent(s2, pl->ev_p1[b], 0)) != cudaSuccess))
             return cuda_fail(e, "slab handoff");
         p2.A = A;
         p2.q_begin = qb;
         p2.q_count = qc;
-        prof_begin(pl, 2, pl->sp[1]);
-        if ((e = fe::launch_phase2(pl->N2, p2, pl->n_ant, pl->sp[1])) != cudaSuccess)
+        prof_begin(pl, 2, s2);
+        if ((e = fe::launch_phase2(pl->N2, p2, pl->n_ant, s2, one)) != cudaSuccess)
             return cuda_fail(e, "phase-2 launch");
-        prof_end(pl, pl->sp[1]);
-        if ((e = cudaEventRecord(pl->ev_p2[b], pl->sp[1])) != cudaSuccess)
+        prof_end(pl, s2);
+        if (!one && (e = cudaEventRecord(pl->ev_p2[b], s2)) != cudaSuccess)
             return cuda_fail(e, "slab event");
     }
     // join: the last phase 2 follows every phase 1 (through the handoff events)
-    if ((e = cudaStreamWaitEvent(st, pl->ev_p2[(pl->n_slabs - 1) & 1], 0)) != cudaSuccess)
+    if (!one && (e = cudaStreamWaitEvent(st, pl->ev_p2[(pl->n_slabs - 1) & 1], 0)) != cudaSuccess)
         return cuda_fail(e, "slab join");
 
-    prof_begin(pl, 3, st);
-    if ((e = fe::launch_tail_update(pl->d_hist[pl->cur], d_packed, pl->d_hist[1 - pl->cur], pl->hist_bytes,
-                                    pl->chunk_bytes, pl->n_streams, st)) != cudaSuccess)
-        return cuda_fail(e, "tail launch");
-    prof_end(pl, st);
     if (pl->profiling) pl->prof_calls++;
     pl->cur = 1 - pl->cur;
     pl->started = true;

@@ -1,7 +1,8 @@
 // Internal declarations shared by the libfengine translation units.
 //
 // Device data path of one fengine_process_chunk call (Sec. 2.1 steps 1-6):
-//   k_delay_table   FP64 delay/phase model per spectrum -> coarse c, fine delta, phase
+//   k_prologue      FP64 delay/phase model per spectrum -> coarse c, fine delta, phase;
+//                   lost-data flags; the last H packed samples of every stream kept
 //   k_phase1<T,N1>  unpack + coarse delay + PFB FIR (Eq. 1) + first FFT stage
 //                   (real N1-point DFT over t1, twiddle by exp(-2 pi i k1 t2 / N))
 //   k_phase2w       1024-point FFT over t2 + fine-delay rotation + gain +
@@ -12,7 +13,6 @@
 // cores: unpack + coarse delay + FIR + first DFT stage with its twiddle in one
 // contraction); the second stage reads its FP16 (FP16 form) or FP32 (BF16
 // form) output.
-//   k_tail_update   keep the last H packed samples of every stream
 // with the four-step split t = N2 t1 + t2, k = k1 + N1 k2 of the 2n-point
 // real DFT (the exp(-2 pi i k1 t2 / N) cross term is the twiddle).
 #pragma once
@@ -20,6 +20,7 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
+#include <type_traits>
 #include <vector>
 
 #include "../../include/fengine.h"
@@ -70,8 +71,6 @@ struct LostDataParams {
     long long m0;
     unsigned char *heap_flags;       // out [ant][ceil(M / S)], nullptr = not wanted
 };
-cudaError_t launch_lost_data(const LostDataParams &p, cudaStream_t s);
-
 struct Phase1Params {
     const uint8_t *chunk;     // [stream][chunk_bytes]
     const uint8_t *hist;      // [stream][hist_bytes], samples [t_in - H, t_in)
@@ -117,13 +116,56 @@ struct Phase2Params {
     float tc_unscale;         // inverse of the power-of-two scale of an FP16 A (1 otherwise)
 };
 
-// Launchers (return cudaGetLastError() of the launch).
-cudaError_t launch_delay_table(const DelayTableParams &p, cudaStream_t s);
+// Launch of a kernel that may begin before the kernel ahead of it in the
+// stream has ended (pdl): it waits for that kernel, complete and its writes
+// visible, at its pdl_wait(). The call's first kernel is launched without, so
+// that everything the caller enqueued before is complete when it starts; every
+// kernel of a call waits for the one before, so that a kernel that has passed
+// its pdl_wait() may use the results of all of them.
+template <class... A>
+inline cudaError_t launch_kernel(void (*k)(A...), dim3 grid, unsigned block, size_t smem, cudaStream_t s, bool pdl,
+                                 const std::common_type_t<A> &...args) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = pdl ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, k, args...);
+}
+#ifdef __CUDACC__
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// the kernel behind this one may begin (its CTAs take what the running ones leave)
+__device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+#endif
+
+// The call's first kernel: the delay table, the lost-data flags (when lost)
+// and the history tail (when tail_bytes), each on its own blocks.
+struct PrologueParams {
+    DelayTableParams d;
+    LostDataParams l;
+    int lost;
+    const uint8_t *hist_in, *chunk;   // [stream][tail_bytes], [stream][chunk_bytes]
+    uint8_t *hist_out;                // [stream][tail_bytes]: the last bytes of [hist_in | chunk]
+    long long tail_bytes, chunk_bytes;
+    int n_streams;
+    int b_delay, b_lost, b_tail;      // blocks of each part (launch_prologue sets them)
+};
+cudaError_t launch_prologue(const PrologueParams &p, cudaStream_t s);
+
+// Launchers (return the launch's error). pdl: see launch_kernel.
 cudaError_t launch_tail_update(const uint8_t *hist_in, const uint8_t *chunk, uint8_t *hist_out,
                                long long hist_bytes, long long chunk_bytes, int n_streams,
                                cudaStream_t s);
-cudaError_t launch_phase1(int T, int N1, const Phase1Params &p, int n_streams, cudaStream_t s);
-cudaError_t launch_phase2(int N2, const Phase2Params &p, int n_ant, cudaStream_t s);
+cudaError_t launch_phase1(int T, int N1, const Phase1Params &p, int n_streams, cudaStream_t s, bool pdl);
+cudaError_t launch_phase2(int N2, const Phase2Params &p, int n_ant, cudaStream_t s, bool pdl);
+// the shared-memory sizes of a plan's kernels (single and grouped), set once on the plan's device
+cudaError_t prepare_phase1(int T, int N1, int W);
+cudaError_t prepare_phase2(int N2, int in);
 
 // ---- grouped launches (batching): the launches of several plans that use
 // one kernel instantiation, as one grid. Member m owns the blocks
@@ -150,7 +192,8 @@ int phase2w_wave();                                                             
 cudaError_t launch_phase1_group(int T, int N1, const Phase1Group &g, cudaStream_t s);
 cudaError_t launch_phase2_group(int N2, int in, const Phase2Group &g, cudaStream_t s);
 // second stage for N2 = 1024 (launch_phase2 and launch_phase2_group route it there)
-cudaError_t launch_phase2w(const Phase2Params &p, int n_ant, cudaStream_t s);
+cudaError_t launch_phase2w(const Phase2Params &p, int n_ant, cudaStream_t s, bool pdl);
+cudaError_t prepare_phase2w(int in);
 cudaError_t launch_phase2w_group(int in, const Phase2Group &g, cudaStream_t s);
 
 // A call of a plan with its phase launches handed back instead of enqueued
@@ -252,8 +295,8 @@ bool phase1_tc_supported(int N, int T, int precision);
 int phase1_tc_phys(int N, int T, int precision);
 void build_phase1_tc_tables(int N, int T, int precision, const float *w, std::vector<uint16_t> &bmat,
                             std::vector<float> &oscale, float &s_int);
-cudaError_t launch_phase1_tc(int T, int precision, const Phase1TcParams &p, cudaStream_t s);
-cudaError_t launch_unpack_cols(const UnpackColsParams &p, cudaStream_t s);
+cudaError_t launch_phase1_tc(int T, int precision, const Phase1TcParams &p, cudaStream_t s, bool pdl);
+cudaError_t launch_unpack_cols(const UnpackColsParams &p, cudaStream_t s, bool pdl);
 // rows of the FP16 column buffer: a call's history + chunk plus the reach of
 // a 128-spectrum pass past the chunk end, padded to a multiple of 64
 inline int unpack_cols_rows(long long H, long long L, long long D, long long Dmin, int N, int T) {

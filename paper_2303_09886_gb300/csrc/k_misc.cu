@@ -1,28 +1,35 @@
-// Small per-call kernels: the FP64 delay/phase table and the history-tail
-// update, plus the phase-1 dispatch over tap counts.
+// The call's first kernel (FP64 delay/phase table, lost-data flags, history
+// tail) and the phase-1 dispatch over tap counts.
 #include "fe_device.cuh"
 #include "fe_internal.cuh"
 
 namespace fe {
 
 template <int T, int CAP>
-cudaError_t launch_phase1_n1(int N1, const GroupArgs<Phase1Params, CAP> &g, cudaStream_t s);
+cudaError_t launch_phase1_n1(int N1, int W, const GroupArgs<Phase1Params, CAP> *g, cudaStream_t s, bool pdl);
 
+// g = nullptr: only the kernel's shared-memory size is set
 template <int CAP>
-static cudaError_t launch_phase1_t(int T, int N1, const GroupArgs<Phase1Params, CAP> &g, cudaStream_t s) {
+static cudaError_t launch_phase1_t(int T, int N1, int W, const GroupArgs<Phase1Params, CAP> *g, cudaStream_t s,
+                                   bool pdl) {
     switch (T) {
-        case 1: return launch_phase1_n1<1, CAP>(N1, g, s);
-        case 2: return launch_phase1_n1<2, CAP>(N1, g, s);
-        case 4: return launch_phase1_n1<4, CAP>(N1, g, s);
-        case 8: return launch_phase1_n1<8, CAP>(N1, g, s);
-        case 16: return launch_phase1_n1<16, CAP>(N1, g, s);
-        case 32: return launch_phase1_n1<32, CAP>(N1, g, s);
+        case 1: return launch_phase1_n1<1, CAP>(N1, W, g, s, pdl);
+        case 2: return launch_phase1_n1<2, CAP>(N1, W, g, s, pdl);
+        case 4: return launch_phase1_n1<4, CAP>(N1, W, g, s, pdl);
+        case 8: return launch_phase1_n1<8, CAP>(N1, W, g, s, pdl);
+        case 16: return launch_phase1_n1<16, CAP>(N1, W, g, s, pdl);
+        case 32: return launch_phase1_n1<32, CAP>(N1, W, g, s, pdl);
         default: return cudaErrorInvalidValue;
     }
 }
 
 cudaError_t launch_phase1_group(int T, int N1, const Phase1Group &g, cudaStream_t s) {
-    return launch_phase1_t<kMaxGroup>(T, N1, g, s);
+    return launch_phase1_t<kMaxGroup>(T, N1, g.p[0].W, &g, s, false);
+}
+
+cudaError_t prepare_phase1(int T, int N1, int W) {
+    const cudaError_t e = launch_phase1_t<1>(T, N1, W, nullptr, nullptr, false);
+    return e != cudaSuccess ? e : launch_phase1_t<kMaxGroup>(T, N1, W, nullptr, nullptr, false);
 }
 
 // blocks of a launch: (t2 blocks, tiles of p.rows spectra, streams)
@@ -33,13 +40,13 @@ int phase1_blocks(int N1, const Phase1Params &p, int n_streams, int *gx, int *gy
     return *gx * *gy * n_streams;
 }
 
-cudaError_t launch_phase1(int T, int N1, const Phase1Params &p, int n_streams, cudaStream_t s) {
+cudaError_t launch_phase1(int T, int N1, const Phase1Params &p, int n_streams, cudaStream_t s, bool pdl) {
     GroupArgs<Phase1Params, 1> g;
     g.p[0] = p;
     g.start[0] = 0;
     g.start[1] = phase1_blocks(N1, p, n_streams, &g.gx, &g.aux[0]);
     g.n = 1;
-    return launch_phase1_t<1>(T, N1, g, s);
+    return launch_phase1_t<1>(T, N1, p.W, &g, s, pdl);
 }
 
 // Spectra per phase-1 CTA. More rows share the T - 1 lead-in rows, the weights
@@ -66,53 +73,51 @@ int phase1_rows(int T, int N1, int N2, int q_count, int n_streams) {
     return best;
 }
 
-// Delay model per spectrum (Sec. 2.1 steps 2 and 4, Sec. 3.3): for the
-// spectrum with timestamp t0 = N m, with the last segment whose t_apply <= t0
-// (segment 0 before all of them),
-//   d = d0 + rate (t0 - t_ref),  c = floor(d + 1/2),  delta = d - c,
-//   phi = phi0 + phi_rate (t0 - t_ref).
+// Delay model of a stream (Sec. 2.1 steps 2 and 4, Sec. 3.3) at the spectrum
+// with timestamp t0 = N m, with the last segment whose t_apply <= t0 (segment
+// 0 before all of them):
+//   d = d0 + rate (t0 - t_ref),  c = floor(d + 1/2),  delta = d - c.
 // FP64 with explicit round-to-nearest operations (no contraction), so the
-// host-side range check in the API computes the very same c. The phase is
+// host-side range check in the API computes the very same c.
+struct DelayAt {
+    long long c;   // clamped into [min_delay, max_delay]
+    bool clamped;
+    double delta, dt;
+    int seg;
+};
+__device__ __forceinline__ DelayAt delay_at(const DelayTableParams &p, int st, long long t0) {
+    const DelaySeg *sg = p.seg + (long long)st * kMaxSeg;
+    const int ns = p.nseg[st];
+    DelayAt r;
+    r.seg = 0;
+    for (int k = 1; k < ns; k++)
+        if (sg[k].t_apply <= t0) r.seg = k;
+    r.dt = (double)(t0 - sg[r.seg].t_ref);
+    const double d = __dadd_rn(sg[r.seg].d0, __dmul_rn(sg[r.seg].rate, r.dt));
+    const double c = floor(__dadd_rn(d, 0.5));
+    r.delta = __dadd_rn(d, -c);
+    r.c = (long long)c;
+    r.clamped = r.c < p.min_delay || r.c > p.max_delay;   // unreachable after the host check
+    if (r.clamped) r.c = r.c < p.min_delay ? p.min_delay : p.max_delay;
+    return r;
+}
+
+// Entry e of the delay table: c, delta and phi = phi0 + phi_rate (t0 - t_ref),
 // reduced to phi/pi in [-1, 1] before the single rounding to FP32.
-__global__ void k_delay_table(const DelayTableParams p) {
-    const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+__device__ __forceinline__ void delay_entry(const DelayTableParams &p, long long e) {
     if (e >= (long long)p.n_streams * p.M) return;
     const int st = (int)(e / p.M), q = (int)(e % p.M);
     const long long t0 = (long long)p.N * (p.m0 + q);
-    const DelaySeg *sg = p.seg + (long long)st * kMaxSeg;
-    const int ns = p.nseg[st];
-    int s = 0;
-    for (int k = 0; k < ns; k++)
-        if (sg[k].t_apply <= t0) s = k;
-    const double dt = (double)(t0 - sg[s].t_ref);
-    const double d = __dadd_rn(sg[s].d0, __dmul_rn(sg[s].rate, dt));
-    const double c = floor(__dadd_rn(d, 0.5));
-    const double delta = __dadd_rn(d, -c);
-    const double phi = __dadd_rn(sg[s].phi0, __dmul_rn(sg[s].phi_rate, dt));
+    const DelayAt a = delay_at(p, st, t0);
+    const DelaySeg &sg = p.seg[(long long)st * kMaxSeg + a.seg];
+    const double phi = __dadd_rn(sg.phi0, __dmul_rn(sg.phi_rate, a.dt));
     const double u = phi * 0.31830988618379067154;       // phi / pi
     const double red = u - 2.0 * rint(0.5 * u);          // in [-1, 1]
-    long long ci = (long long)c;
-    if (ci < p.min_delay || ci > p.max_delay) {          // unreachable after the host check
-        ci = ci < p.min_delay ? p.min_delay : p.max_delay;
-        atomicExch(p.err, 1);
-    }
-    p.ctab[e] = (int)ci;
-    p.ftab[e] = make_float2((float)delta, (float)red);
-    if (p.cchg) {
-        // the previous spectrum's coarse delay, recomputed the same way
-        int chg = 0;
-        if (q > 0) {
-            const long long tp = t0 - p.N;
-            int sp = 0;
-            for (int k = 0; k < ns; k++)
-                if (sg[k].t_apply <= tp) sp = k;
-            const double dp = __dadd_rn(sg[sp].d0, __dmul_rn(sg[sp].rate, (double)(tp - sg[sp].t_ref)));
-            long long cp = (long long)floor(__dadd_rn(dp, 0.5));
-            cp = cp < p.min_delay ? p.min_delay : (cp > p.max_delay ? p.max_delay : cp);
-            chg = cp != ci;
-        }
-        p.cchg[e] = (unsigned char)chg;
-    }
+    if (a.clamped) atomicExch(p.err, 1);
+    p.ctab[e] = (int)a.c;
+    p.ftab[e] = make_float2((float)a.delta, (float)red);
+    // the previous spectrum's coarse delay, recomputed the same way
+    if (p.cchg) p.cchg[e] = (unsigned char)(q > 0 && delay_at(p, st, t0 - p.N).c != a.c);
     if (p.g_tapply) {
         const long long *ta = p.g_tapply + (long long)st * kMaxGainSeg;
         int g = 0;
@@ -122,40 +127,24 @@ __global__ void k_delay_table(const DelayTableParams p) {
     }
 }
 
-cudaError_t launch_delay_table(const DelayTableParams &p, cudaStream_t s) {
-    const long long total = (long long)p.n_streams * p.M;
-    const int threads = 256;
-    const long long blocks = (total + threads - 1) / threads;
-    k_delay_table<<<(unsigned)blocks, threads, 0, s>>>(p);
-    return cudaGetLastError();
-}
-
-// New history = the last hist_bytes bytes of [old history | chunk] for every
-// stream (the chunk-overlap region of Sec. 3.1, kept resident on the device
-// instead of copying the next chunk's prefix).
-__global__ void k_tail_update(const uint8_t *__restrict__ hist_in, const uint8_t *__restrict__ chunk,
-                              uint8_t *__restrict__ hist_out, long long hist_bytes,
-                              long long chunk_bytes, int n_streams) {
-    const long long total = hist_bytes * n_streams;
-    for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < total;
-         e += (long long)gridDim.x * blockDim.x) {
-        const long long st = e / hist_bytes, b = e % hist_bytes;
-        const long long src = b + chunk_bytes;
-        hist_out[e] = src < hist_bytes ? hist_in[st * hist_bytes + src]
-                                       : chunk[st * chunk_bytes + (src - hist_bytes)];
+// History tail: word w of the new history (32-bit words; every stream's bytes
+// are a multiple of 4 and 4-byte aligned): the last tail_bytes bytes of [old
+// history | chunk] of every stream (the chunk-overlap region of Sec. 3.1, kept
+// resident on the device instead of copying the next chunk's prefix).
+__device__ __forceinline__ void tail_words(const uint8_t *hist_in, const uint8_t *chunk, uint8_t *hist_out,
+                                           long long tail_bytes, long long chunk_bytes, int n_streams, int block,
+                                           int n_blocks) {
+    const unsigned tw = (unsigned)(tail_bytes >> 2), cw = (unsigned)(chunk_bytes >> 2);
+    const uint32_t *hi = reinterpret_cast<const uint32_t *>(hist_in), *ch = reinterpret_cast<const uint32_t *>(chunk);
+    uint32_t *ho = reinterpret_cast<uint32_t *>(hist_out);
+    for (int st = 0; st < n_streams; st++) {
+        const uint32_t *h = hi + (long long)st * tw, *c = ch + (long long)st * cw;
+        uint32_t *o = ho + (long long)st * tw;
+        for (unsigned w = (unsigned)block * blockDim.x + threadIdx.x; w < tw; w += (unsigned)n_blocks * blockDim.x) {
+            const unsigned src = w + cw;
+            o[w] = src < tw ? h[src] : c[src - tw];
+        }
     }
-}
-
-cudaError_t launch_tail_update(const uint8_t *hist_in, const uint8_t *chunk, uint8_t *hist_out,
-                               long long hist_bytes, long long chunk_bytes, int n_streams,
-                               cudaStream_t s) {
-    const long long total = hist_bytes * n_streams;
-    long long blocks = (total + 255) / 256;
-    if (blocks > 4096) blocks = 4096;
-    if (blocks < 1) blocks = 1;
-    k_tail_update<<<(unsigned)blocks, 256, 0, s>>>(hist_in, chunk, hist_out, hist_bytes, chunk_bytes,
-                                                   n_streams);
-    return cudaGetLastError();
 }
 
 // Lost data (Sec. 3.7). Block x < n_ant * n_heaps_out: output heap h of
@@ -165,7 +154,7 @@ cudaError_t launch_tail_update(const uint8_t *hist_in, const uint8_t *chunk, uin
 // heaps from valid). The heap is transmitted (flag 1) iff all are usable.
 // The last block writes the received flags of the HV heaps before the end
 // of this chunk, for the next call.
-__global__ void k_lost_data(const LostDataParams p) {
+__device__ __forceinline__ void lost_block(const LostDataParams &p, const DelayTableParams &d, int block) {
     const int n_out = (p.M + p.S - 1) / p.S;
     const long long hist_first = p.heap0 - p.HV;   // heap of hv_in[0]
     auto received = [&](int stream, long long h) -> bool {
@@ -177,14 +166,14 @@ __global__ void k_lost_data(const LostDataParams p) {
         const long long i = h - hist_first;
         return i >= 0 && p.hv_in[(long long)stream * p.HV + i] != 0;
     };
-    if ((int)blockIdx.x < p.n_ant * n_out) {
+    if (block < p.n_ant * n_out) {
         if (!p.heap_flags) return;
-        const int a = blockIdx.x / n_out, h = blockIdx.x % n_out;
+        const int a = block / n_out, h = block % n_out;
         const int q0 = h * p.S, cnt = min(p.S, p.M - q0);
         int ok = 1;
         for (int e = threadIdx.x; e < 2 * cnt; e += blockDim.x) {
             const int pol = e / cnt, q = q0 + e % cnt, stream = 2 * a + pol;
-            const long long start = (long long)p.N * (p.m0 + q) - p.ctab[(long long)stream * p.M + q];
+            const long long start = (long long)p.N * (p.m0 + q) - delay_at(d, stream, (long long)p.N * (p.m0 + q)).c;
             const long long end = start + (long long)p.N * p.T - 1;
             const long long h0 = start >= 0 ? start / kHeapSamples : -((-start + kHeapSamples - 1) / kHeapSamples);
             const long long h1 = end >= 0 ? end / kHeapSamples : -((-end + kHeapSamples - 1) / kHeapSamples);
@@ -203,10 +192,43 @@ __global__ void k_lost_data(const LostDataParams p) {
     }
 }
 
-cudaError_t launch_lost_data(const LostDataParams &p, cudaStream_t s) {
-    const int n_out = (p.M + p.S - 1) / p.S;
-    k_lost_data<<<p.n_ant * n_out + 1, 256, 0, s>>>(p);
-    return cudaGetLastError();
+__global__ void __launch_bounds__(256) k_prologue(const __grid_constant__ PrologueParams p) {
+    pdl_release();
+    const int b = (int)blockIdx.x;
+    if (b < p.b_delay) {
+        delay_entry(p.d, (long long)b * 256 + threadIdx.x);
+    } else if (b < p.b_delay + p.b_lost) {
+        lost_block(p.l, p.d, b - p.b_delay);
+    } else {
+        tail_words(p.hist_in, p.chunk, p.hist_out, p.tail_bytes, p.chunk_bytes, p.n_streams, b - p.b_delay - p.b_lost,
+                   p.b_tail);
+    }
+}
+
+// blocks of a history tail: about 8 words per thread over all streams, at most 4 blocks per SM
+static int tail_blocks(long long tail_bytes, int n_streams) {
+    const long long per = (tail_bytes / 4 + 255) / 256, want = (per * n_streams + 7) / 8;
+    return (int)(want < 1 ? 1 : want > per ? (per < 608 ? per : 608) : want > 608 ? 608 : want);
+}
+
+cudaError_t launch_prologue(const PrologueParams &q, cudaStream_t s) {
+    PrologueParams p = q;
+    p.b_delay = (int)(((long long)p.d.n_streams * p.d.M + 255) / 256);
+    p.b_lost = p.lost ? p.l.n_ant * ((p.l.M + p.l.S - 1) / p.l.S) + 1 : 0;
+    p.b_tail = p.tail_bytes > 0 ? tail_blocks(p.tail_bytes, p.n_streams) : 0;
+    return launch_kernel(k_prologue, dim3((unsigned)(p.b_delay + p.b_lost + p.b_tail)), 256u, 0, s, false, p);
+}
+
+// The history tail by itself (the down-converter's).
+__global__ void __launch_bounds__(256) k_tail_update(const uint8_t *hist_in, const uint8_t *chunk, uint8_t *hist_out,
+                                                     long long tail_bytes, long long chunk_bytes, int n_streams) {
+    tail_words(hist_in, chunk, hist_out, tail_bytes, chunk_bytes, n_streams, (int)blockIdx.x, (int)gridDim.x);
+}
+
+cudaError_t launch_tail_update(const uint8_t *hist_in, const uint8_t *chunk, uint8_t *hist_out, long long hist_bytes,
+                               long long chunk_bytes, int n_streams, cudaStream_t s) {
+    return launch_kernel(k_tail_update, dim3((unsigned)tail_blocks(hist_bytes, n_streams)), 256u, 0, s, false, hist_in, chunk,
+                         hist_out, hist_bytes, chunk_bytes, n_streams);
 }
 
 }  // namespace fe

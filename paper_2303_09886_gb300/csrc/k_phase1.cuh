@@ -392,6 +392,15 @@ __global__ void __launch_bounds__(kP1Threads, 2) k_phase1(const __grid_constant_
     // sample (from the first history sample) of input row 0, column t = 0, before the delay
     const long long rel_base = (long long)N * (p.m0 + q0) - (p.t_in - p.H) + t2_0;
 
+    // this tile's twiddles exp(-2 pi i k1 t2 / N) (read after the first block's barrier)
+    for (int i = threadIdx.x; i < (N1 / 2 + 1) * W; i += kP1Threads) {
+        const float2 v = __ldg(p.tw1 + (long long)(i / W) * N2 + t2_0 + i % W);
+        if constexpr (S::PAIR) reinterpret_cast<float4 *>(tw)[i] = make_float4(v.x, v.x, v.y, v.y);
+        else reinterpret_cast<float2 *>(tw)[i] = v;
+    }
+    pdl_release();
+    pdl_wait();
+
     // the coarse delay of each block (lane i: output row i), and whether its rows share it
     const int nblk = (Rv + kP1Block - 1) / kP1Block;
     int cdl[kP1Blocks];
@@ -406,13 +415,6 @@ __global__ void __launch_bounds__(kP1Threads, 2) k_phase1(const __grid_constant_
     const bool filt = c < S::C, fwarp = warp < S::NW;   // (a tile of 32 columns fills half a warp)
     const int t = N2 * (c / W) + (c % W);   // column offset in a row
     const float *wcol = p.w + t2_0 + (filt ? t : 0);
-    // this tile's twiddles exp(-2 pi i k1 t2 / N) (read after the first block's barrier)
-    for (int i = threadIdx.x; i < (N1 / 2 + 1) * W; i += kP1Threads) {
-        const float2 v = __ldg(p.tw1 + (long long)(i / W) * N2 + t2_0 + i % W);
-        if constexpr (S::PAIR) reinterpret_cast<float4 *>(tw)[i] = make_float4(v.x, v.x, v.y, v.y);
-        else reinterpret_cast<float2 *>(tw)[i] = v;
-    }
-
     P1Stage<T, N1, W> st;
     st.chunk0 = chunk - p.hist_bytes;
     st.hist = hist;
@@ -539,33 +541,32 @@ __global__ void __launch_bounds__(kP1Threads, 2) k_phase1(const __grid_constant_
     }
 }
 
+// (g = nullptr: only the kernel's shared-memory size is set)
 template <int T, int N1, int W, int CAP>
-cudaError_t launch_phase1_tw(const GroupArgs<Phase1Params, CAP> &g, cudaStream_t s) {
+cudaError_t launch_phase1_tw(const GroupArgs<Phase1Params, CAP> *g, cudaStream_t s, bool pdl) {
     using S = P1Shape<T, N1, W>;
     static_assert(kP1Block % S::RING == 0, "a row's ring slot is the same in every block");
-    cudaError_t e =
-        cudaFuncSetAttribute(k_phase1<T, N1, W, CAP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::SMEM);
-    if (e != cudaSuccess) return e;
-    for (int m = 0; m < g.n; m++)
-        if (g.p[m].W != W || g.p[m].N2 % W || g.p[m].rows < 1 || g.p[m].rows > kP1Blocks * kP1Block ||
-            (g.p[m].rows & 1))
+    if (!g)
+        return cudaFuncSetAttribute(k_phase1<T, N1, W, CAP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::SMEM);
+    for (int m = 0; m < g->n; m++)
+        if (g->p[m].W != W || g->p[m].N2 % W || g->p[m].rows < 1 || g->p[m].rows > kP1Blocks * kP1Block ||
+            (g->p[m].rows & 1))
             return cudaErrorInvalidValue;
-    if (g.n < 1 || g.start[g.n] < 1) return cudaSuccess;
-    k_phase1<T, N1, W, CAP><<<g.start[g.n], kP1Threads, S::SMEM, s>>>(g);
-    return cudaGetLastError();
+    if (g->n < 1 || g->start[g->n] < 1) return cudaSuccess;
+    return launch_kernel(k_phase1<T, N1, W, CAP>, dim3((unsigned)g->start[g->n]), (unsigned)kP1Threads, S::SMEM, s, pdl, *g);
 }
 
 template <int T, int CAP>
-cudaError_t launch_phase1_n1(int N1, const GroupArgs<Phase1Params, CAP> &g, cudaStream_t s) {
-    switch (N1 * 1000 + g.p[0].W) {
-        case 8064: return launch_phase1_tw<T, 8, 64, CAP>(g, s);
-        case 16032: return launch_phase1_tw<T, 16, 32, CAP>(g, s);
-        case 32016: return launch_phase1_tw<T, 32, 16, CAP>(g, s);
-        case 64008: return launch_phase1_tw<T, 64, 8, CAP>(g, s);
-        case 8032: return launch_phase1_tw<T, 8, 32, CAP>(g, s);
-        case 8016: return launch_phase1_tw<T, 8, 16, CAP>(g, s);
-        case 8008: return launch_phase1_tw<T, 8, 8, CAP>(g, s);
-        case 8004: return launch_phase1_tw<T, 8, 4, CAP>(g, s);
+cudaError_t launch_phase1_n1(int N1, int W, const GroupArgs<Phase1Params, CAP> *g, cudaStream_t s, bool pdl) {
+    switch (N1 * 1000 + W) {
+        case 8064: return launch_phase1_tw<T, 8, 64, CAP>(g, s, pdl);
+        case 16032: return launch_phase1_tw<T, 16, 32, CAP>(g, s, pdl);
+        case 32016: return launch_phase1_tw<T, 32, 16, CAP>(g, s, pdl);
+        case 64008: return launch_phase1_tw<T, 64, 8, CAP>(g, s, pdl);
+        case 8032: return launch_phase1_tw<T, 8, 32, CAP>(g, s, pdl);
+        case 8016: return launch_phase1_tw<T, 8, 16, CAP>(g, s, pdl);
+        case 8008: return launch_phase1_tw<T, 8, 8, CAP>(g, s, pdl);
+        case 8004: return launch_phase1_tw<T, 8, 4, CAP>(g, s, pdl);
         default: return cudaErrorInvalidValue;
     }
 }

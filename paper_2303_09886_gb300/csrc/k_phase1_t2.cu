@@ -3,6 +3,6 @@
 #include "k_phase1.cuh"
 
 namespace fe {
-template cudaError_t launch_phase1_n1<2, 1>(int, const GroupArgs<Phase1Params, 1> &, cudaStream_t);
-template cudaError_t launch_phase1_n1<2, kMaxGroup>(int, const Phase1Group &, cudaStream_t);
+template cudaError_t launch_phase1_n1<2, 1>(int, int, const GroupArgs<Phase1Params, 1> *, cudaStream_t, bool);
+template cudaError_t launch_phase1_n1<2, kMaxGroup>(int, int, const Phase1Group *, cudaStream_t, bool);
 }  // namespace fe

@@ -291,6 +291,8 @@ __global__ void __launch_bounds__(256) k_unpack_cols(const UnpackColsParams p) {
     __shared__ uint32_t tile[64][33];    // [column][row pair] FP16 pairs
     const int col0 = blockIdx.x * 64, r0 = p.row_begin + blockIdx.y * 64, st = blockIdx.z;
     const int tid = threadIdx.x;
+    pdl_release();
+    pdl_wait();
     const long long c0 = p.ctab[(long long)st * p.M];
     // relative sample (from the first history sample) of row 0, column col0;
     // history and chunk are one bit stream (10 H is a multiple of 32)
@@ -369,6 +371,8 @@ __global__ void __launch_bounds__(256) k_unpack_cols(const UnpackColsParams p) {
 // The same for P < 64 (n_channels < 256): one thread per output sample,
 // read as two bytes of the packed stream.
 __global__ void k_unpack_cols_small(const UnpackColsParams p) {
+    pdl_release();
+    pdl_wait();
     const long long total = (long long)p.n_streams * p.P * p.RTP;
     for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < total;
          e += (long long)gridDim.x * blockDim.x) {
@@ -464,6 +468,8 @@ __global__ void __launch_bounds__(tc_threads(tc_one_cta(PH, R, T, PREC)), tc_one
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
+    pdl_release();
+    pdl_wait();   // the columns and the delay table
 
     // a bounded wait that also gives up once another role has
     auto wait_bar = [&](unsigned long long *b, uint32_t parity) -> bool {
@@ -879,7 +885,7 @@ void build_phase1_tc_tables(int N, int T, int precision, const float *w, std::ve
 }
 
 template <int R, int T, int PREC, int PH>
-static cudaError_t launch_tc_ph(const Phase1TcParams &p, cudaStream_t s) {
+static cudaError_t launch_tc_ph(const Phase1TcParams &p, cudaStream_t s, bool pdl) {
     const size_t smem = tc_smem_bytes(PH, R, T, PREC);
     cudaError_t e = cudaFuncSetAttribute(k_phase1_tc<R, T, PREC, PH>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)smem);
@@ -891,48 +897,48 @@ static cudaError_t launch_tc_ph(const Phase1TcParams &p, cudaStream_t s) {
     const long long ctas = (long long)p.splits * (tc_one_cta(PH, R, T, PREC) ? 1 : 2);
     const int grid = (int)(n_units < ctas ? n_units : ctas);
     if (grid < 1) return cudaErrorInvalidValue;
-    k_phase1_tc<R, T, PREC, PH><<<grid, tc_threads(tc_one_cta(PH, R, T, PREC)), smem, s>>>(p);
-    return cudaGetLastError();
+    return launch_kernel(k_phase1_tc<R, T, PREC, PH>, dim3((unsigned)grid),
+                         (unsigned)tc_threads(tc_one_cta(PH, R, T, PREC)), smem, s, pdl, p);
 }
 
 // the kernel with the column count phase1_tc_phys gives for this N
 template <int R, int T, int PREC>
-static cudaError_t launch_tc(const Phase1TcParams &p, cudaStream_t s) {
+static cudaError_t launch_tc(const Phase1TcParams &p, cudaStream_t s, bool pdl) {
     if constexpr (tc_phys(R, T, PREC) == 16) {
         if constexpr (R == 1) {
-            if (p.N2 < 16) return launch_tc_ph<R, T, PREC, 8>(p, s);
+            if (p.N2 < 16) return launch_tc_ph<R, T, PREC, 8>(p, s, pdl);
         }
-        return launch_tc_ph<R, T, PREC, 16>(p, s);
+        return launch_tc_ph<R, T, PREC, 16>(p, s, pdl);
     } else {
-        return launch_tc_ph<R, T, PREC, 8>(p, s);
+        return launch_tc_ph<R, T, PREC, 8>(p, s, pdl);
     }
 }
 
 template <int R, int PREC>
-static cudaError_t launch_tc_t(int T, const Phase1TcParams &p, cudaStream_t s) {
+static cudaError_t launch_tc_t(int T, const Phase1TcParams &p, cudaStream_t s, bool pdl) {
     switch (T) {
-        case 1: return launch_tc<R, 1, PREC>(p, s);
-        case 2: return launch_tc<R, 2, PREC>(p, s);
-        case 4: return launch_tc<R, 4, PREC>(p, s);
-        case 8: return launch_tc<R, 8, PREC>(p, s);
-        case 16: return launch_tc<R, 16, PREC>(p, s);
-        case 32: return launch_tc<R, 32, PREC>(p, s);
+        case 1: return launch_tc<R, 1, PREC>(p, s, pdl);
+        case 2: return launch_tc<R, 2, PREC>(p, s, pdl);
+        case 4: return launch_tc<R, 4, PREC>(p, s, pdl);
+        case 8: return launch_tc<R, 8, PREC>(p, s, pdl);
+        case 16: return launch_tc<R, 16, PREC>(p, s, pdl);
+        case 32: return launch_tc<R, 32, PREC>(p, s, pdl);
         default: return cudaErrorInvalidValue;
     }
 }
 
 template <int PREC>
-static cudaError_t launch_tc_r(int R, int T, const Phase1TcParams &p, cudaStream_t s) {
+static cudaError_t launch_tc_r(int R, int T, const Phase1TcParams &p, cudaStream_t s, bool pdl) {
     switch (R) {
-        case 1: return launch_tc_t<1, PREC>(T, p, s);
-        case 2: return launch_tc_t<2, PREC>(T, p, s);
-        case 4: return launch_tc_t<4, PREC>(T, p, s);
-        case 8: return launch_tc_t<8, PREC>(T, p, s);
+        case 1: return launch_tc_t<1, PREC>(T, p, s, pdl);
+        case 2: return launch_tc_t<2, PREC>(T, p, s, pdl);
+        case 4: return launch_tc_t<4, PREC>(T, p, s, pdl);
+        case 8: return launch_tc_t<8, PREC>(T, p, s, pdl);
         default: return cudaErrorInvalidValue;
     }
 }
 
-cudaError_t launch_unpack_cols(const UnpackColsParams &p, cudaStream_t s) {
+cudaError_t launch_unpack_cols(const UnpackColsParams &p, cudaStream_t s, bool pdl) {
     if (p.RTP % 64) return cudaErrorInvalidValue;
     if (p.row_begin % 64 || p.row_end % 64 || p.row_begin < 0 || p.row_end > p.RTP || p.row_end < p.row_begin)
         return cudaErrorInvalidValue;
@@ -941,18 +947,17 @@ cudaError_t launch_unpack_cols(const UnpackColsParams &p, cudaStream_t s) {
         if (p.row_begin != 0 || p.row_end != p.RTP) return cudaErrorInvalidValue;   // whole buffer only
         const long long total = (long long)p.n_streams * p.P * p.RTP;
         const long long blocks = (total + 255) / 256 < 8192 ? (total + 255) / 256 : 8192;
-        k_unpack_cols_small<<<(unsigned)blocks, 256, 0, s>>>(p);
+        return launch_kernel(k_unpack_cols_small, dim3((unsigned)blocks), 256u, 0, s, pdl, p);
     } else {
         dim3 grid(p.P / 64, (p.row_end - p.row_begin) / 64, p.n_streams);
-        k_unpack_cols<<<grid, 256, 0, s>>>(p);
+        return launch_kernel(k_unpack_cols, grid, 256u, 0, s, pdl, p);
     }
-    return cudaGetLastError();
 }
 
-cudaError_t launch_phase1_tc(int T, int precision, const Phase1TcParams &p, cudaStream_t s) {
+cudaError_t launch_phase1_tc(int T, int precision, const Phase1TcParams &p, cudaStream_t s, bool pdl) {
     if (p.q_count <= 0) return cudaSuccess;
     const int R = phase1_tc_R(p.N);
-    return precision == 2 ? launch_tc_r<2>(R, T, p, s) : launch_tc_r<1>(R, T, p, s);
+    return precision == 2 ? launch_tc_r<2>(R, T, p, s, pdl) : launch_tc_r<1>(R, T, p, s, pdl);
 }
 
 }  // namespace fe

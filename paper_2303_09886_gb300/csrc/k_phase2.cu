@@ -176,6 +176,8 @@ __global__ void __launch_bounds__(kP2Threads, 3) k_phase2(const __grid_constant_
 
     const int k1 = blk % ga.gx, ant = blk / (ga.gx * gy);
     const int q0 = p.q_begin + ((blk / ga.gx) % gy) * R2;
+    pdl_release();
+    pdl_wait();
 #include "k_phase2_tile.inc"
 }
 
@@ -194,57 +196,61 @@ int phase2_blocks(int N2, const Phase2Params &p, int n_ant, int *gx, int *gy) {
     return *gx * *gy * n_ant;
 }
 
+// (g = nullptr: only the kernel's shared-memory size is set)
 template <int N2, int IN, int CAP>
-static cudaError_t launch_p2(const GroupArgs<Phase2Params, CAP> &g, cudaStream_t s) {
+static cudaError_t launch_p2(const GroupArgs<Phase2Params, CAP> *g, cudaStream_t s, bool pdl) {
     const int R2 = P2Shape<N2>::R2;
     const size_t smem = phase2_smem_bytes(N2, R2);
-    cudaError_t e =
-        cudaFuncSetAttribute(k_phase2<N2, IN, CAP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    for (int m = 0; m < g.n; m++)
-        if (g.p[m].R2 != R2 || g.p[m].a_spectra % 2) return cudaErrorInvalidValue;
-    if (g.n < 1 || g.start[g.n] < 1) return cudaSuccess;
-    k_phase2<N2, IN, CAP><<<g.start[g.n], kP2Threads, smem, s>>>(g);
-    return cudaGetLastError();
+    if (!g) return cudaFuncSetAttribute(k_phase2<N2, IN, CAP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    for (int m = 0; m < g->n; m++)
+        if (g->p[m].R2 != R2 || g->p[m].a_spectra % 2) return cudaErrorInvalidValue;
+    if (g->n < 1 || g->start[g->n] < 1) return cudaSuccess;
+    return launch_kernel(k_phase2<N2, IN, CAP>, dim3((unsigned)g->start[g->n]), (unsigned)kP2Threads, smem, s, pdl, *g);
 }
 
 template <int N2, int CAP>
-static cudaError_t launch_p2_in(int in, const GroupArgs<Phase2Params, CAP> &g, cudaStream_t s) {
+static cudaError_t launch_p2_in(int in, const GroupArgs<Phase2Params, CAP> *g, cudaStream_t s, bool pdl) {
     switch (in) {
-        case kInPairs: return launch_p2<N2, kInPairs, CAP>(g, s);
-        case kInHalf: return launch_p2<N2, kInHalf, CAP>(g, s);
-        default: return launch_p2<N2, kInFloat, CAP>(g, s);
+        case kInPairs: return launch_p2<N2, kInPairs, CAP>(g, s, pdl);
+        case kInHalf: return launch_p2<N2, kInHalf, CAP>(g, s, pdl);
+        default: return launch_p2<N2, kInFloat, CAP>(g, s, pdl);
     }
 }
 
 template <int CAP>
-static cudaError_t launch_p2_n2(int N2, int in, const GroupArgs<Phase2Params, CAP> &g, cudaStream_t s) {
+static cudaError_t launch_p2_n2(int N2, int in, const GroupArgs<Phase2Params, CAP> *g, cudaStream_t s, bool pdl) {
     switch (N2) {
-        case 2: return launch_p2_in<2>(in, g, s);
-        case 4: return launch_p2_in<4>(in, g, s);
-        case 8: return launch_p2_in<8>(in, g, s);
-        case 16: return launch_p2_in<16>(in, g, s);
-        case 32: return launch_p2_in<32>(in, g, s);
-        case 64: return launch_p2_in<64>(in, g, s);
-        case 128: return launch_p2_in<128>(in, g, s);
-        case 256: return launch_p2_in<256>(in, g, s);
-        case 512: return launch_p2_in<512>(in, g, s);
+        case 2: return launch_p2_in<2, CAP>(in, g, s, pdl);
+        case 4: return launch_p2_in<4, CAP>(in, g, s, pdl);
+        case 8: return launch_p2_in<8, CAP>(in, g, s, pdl);
+        case 16: return launch_p2_in<16, CAP>(in, g, s, pdl);
+        case 32: return launch_p2_in<32, CAP>(in, g, s, pdl);
+        case 64: return launch_p2_in<64, CAP>(in, g, s, pdl);
+        case 128: return launch_p2_in<128, CAP>(in, g, s, pdl);
+        case 256: return launch_p2_in<256, CAP>(in, g, s, pdl);
+        case 512: return launch_p2_in<512, CAP>(in, g, s, pdl);
         default: return cudaErrorInvalidValue;
     }
 }
 
-cudaError_t launch_phase2_group(int N2, int in, const Phase2Group &g, cudaStream_t s) {
-    return N2 == 1024 ? launch_phase2w_group(in, g, s) : launch_p2_n2(N2, in, g, s);
+cudaError_t prepare_phase2(int N2, int in) {
+    if (N2 == 1024) return prepare_phase2w(in);
+    const cudaError_t e = launch_p2_n2<1>(N2, in, nullptr, nullptr, false);
+    return e != cudaSuccess ? e : launch_p2_n2<kMaxGroup>(N2, in, nullptr, nullptr, false);
 }
 
-cudaError_t launch_phase2(int N2, const Phase2Params &p, int n_ant, cudaStream_t s) {
-    if (N2 == 1024) return launch_phase2w(p, n_ant, s);   // one warp per pair of 1024-point sequences
+cudaError_t launch_phase2_group(int N2, int in, const Phase2Group &g, cudaStream_t s) {
+    return N2 == 1024 ? launch_phase2w_group(in, g, s) : launch_p2_n2(N2, in, &g, s, false);
+}
+
+cudaError_t launch_phase2(int N2, const Phase2Params &p, int n_ant, cudaStream_t s, bool pdl) {
+    if (N2 == 1024) return launch_phase2w(p, n_ant, s, pdl);   // one warp per pair of 1024-point sequences
     GroupArgs<Phase2Params, 1> g;
     g.p[0] = p;
     g.start[0] = 0;
     g.start[1] = phase2_blocks(N2, p, n_ant, &g.gx, &g.aux[0]);
     g.n = 1;
-    return launch_p2_n2(N2, p.in, g, s);
+    return launch_p2_n2(N2, p.in, &g, s, pdl);
 }
 
 }  // namespace fe

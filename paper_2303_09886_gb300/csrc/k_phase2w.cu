@@ -204,15 +204,17 @@ __global__ void __launch_bounds__(kWThreads, 1) k_phase2w(const __grid_constant_
         f1 = __ldg(p.ftab + sq + q1);
         if (p.gsel) gsel = (int)__ldg(p.gsel + sq + q) | (int)__ldg(p.gsel + sq + q1) << 8;
     };
+    for (int e = threadIdx.x; e < 32 * 32; e += kWThreads) {
+        const float2 t = __ldg(p.tw2 + (((e >> 5) * (e & 31)) & (kWN2 - 1)));
+        (&sm.tw[0][0])[e] = make_float4(t.x, t.x, t.y, t.y);
+    }
+    pdl_release();
+    pdl_wait();   // phase 1's results, and the delay table's
     if (it0 + grp < it1 && active_in(nx)) {
         if (lane == 0) fetch(nx);
         model(nx);
     }
     uint32_t parity = 0;
-    for (int e = threadIdx.x; e < 32 * 32; e += kWThreads) {
-        const float2 t = __ldg(p.tw2 + (((e >> 5) * (e & 31)) & (kWN2 - 1)));
-        (&sm.tw[0][0])[e] = make_float4(t.x, t.x, t.y, t.y);
-    }
 
     for (int seg = it0; seg < it1;) {
         // [seg, se): items of one class and antenna whose first spectra use the same gain sets
@@ -456,30 +458,34 @@ int phase2w_wave() {
     return sms;
 }
 
+// (g = nullptr: only the kernel's shared-memory size is set)
 template <int IN, int CAP>
-static cudaError_t launch_w(const GroupArgs<Phase2Params, CAP> &g, cudaStream_t s) {
-    cudaError_t e =
-        cudaFuncSetAttribute(k_phase2w<IN, CAP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(WSmem));
-    if (e != cudaSuccess) return e;
-    for (int m = 0; m < g.n; m++)
-        if (g.p[m].N / g.p[m].N1 != kWN2 || g.p[m].a_spectra % 2) return cudaErrorInvalidValue;
-    if (g.n < 1 || g.start[g.n] < 1) return cudaSuccess;
-    k_phase2w<IN, CAP><<<g.start[g.n], kWThreads, sizeof(WSmem), s>>>(g);
-    return cudaGetLastError();
+static cudaError_t launch_w(const GroupArgs<Phase2Params, CAP> *g, cudaStream_t s, bool pdl) {
+    if (!g)
+        return cudaFuncSetAttribute(k_phase2w<IN, CAP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(WSmem));
+    for (int m = 0; m < g->n; m++)
+        if (g->p[m].N / g->p[m].N1 != kWN2 || g->p[m].a_spectra % 2) return cudaErrorInvalidValue;
+    if (g->n < 1 || g->start[g->n] < 1) return cudaSuccess;
+    return launch_kernel(k_phase2w<IN, CAP>, dim3((unsigned)g->start[g->n]), (unsigned)kWThreads, sizeof(WSmem), s, pdl, *g);
 }
 
 template <int CAP>
-static cudaError_t launch_w_in(int in, const GroupArgs<Phase2Params, CAP> &g, cudaStream_t s) {
+static cudaError_t launch_w_in(int in, const GroupArgs<Phase2Params, CAP> *g, cudaStream_t s, bool pdl) {
     switch (in) {
-        case kInPairs: return launch_w<kInPairs, CAP>(g, s);
-        case kInHalf: return launch_w<kInHalf, CAP>(g, s);
-        default: return launch_w<kInFloat, CAP>(g, s);
+        case kInPairs: return launch_w<kInPairs, CAP>(g, s, pdl);
+        case kInHalf: return launch_w<kInHalf, CAP>(g, s, pdl);
+        default: return launch_w<kInFloat, CAP>(g, s, pdl);
     }
 }
 
-cudaError_t launch_phase2w_group(int in, const Phase2Group &g, cudaStream_t s) { return launch_w_in(in, g, s); }
+cudaError_t prepare_phase2w(int in) {
+    const cudaError_t e = launch_w_in<1>(in, nullptr, nullptr, false);
+    return e != cudaSuccess ? e : launch_w_in<kMaxGroup>(in, nullptr, nullptr, false);
+}
 
-cudaError_t launch_phase2w(const Phase2Params &p, int n_ant, cudaStream_t s) {
+cudaError_t launch_phase2w_group(int in, const Phase2Group &g, cudaStream_t s) { return launch_w_in(in, &g, s, false); }
+
+cudaError_t launch_phase2w(const Phase2Params &p, int n_ant, cudaStream_t s, bool pdl) {
     const long long items = phase2w_items(p, n_ant);
     if (items <= 0) return cudaSuccess;
     const int wave = phase2w_wave();
@@ -491,7 +497,7 @@ cudaError_t launch_phase2w(const Phase2Params &p, int n_ant, cudaStream_t s) {
     g.aux[0] = n_ant;
     g.gx = 1;
     g.n = 1;
-    return launch_w_in(p.in, g, s);
+    return launch_w_in(p.in, &g, s, pdl);
 }
 
 }  // namespace fe

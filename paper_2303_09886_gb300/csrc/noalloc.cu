@@ -188,7 +188,9 @@ fengine_status fengine_process_chunk_noalloc(const fengine_noalloc_args *a, cons
     dp.ctab = reinterpret_cast<int *>(base + o_ctab);
     dp.ftab = reinterpret_cast<float2 *>(base + o_ftab);
     dp.err = reinterpret_cast<int *>(base + o_err);
-    if (fe::launch_delay_table(dp, st) != cudaSuccess) return FENGINE_ECUDA;
+    fe::PrologueParams pp{};
+    pp.d = dp;
+    if (fe::launch_prologue(pp, st) != cudaSuccess) return FENGINE_ECUDA;
 
     fe::Phase1Params p1{};
     p1.chunk = d_packed;
@@ -229,14 +231,17 @@ fengine_status fengine_process_chunk_noalloc(const fengine_noalloc_args *a, cons
     p2.in = fe::phase1_layout(N1);
     p2.a_spectra = (int)SL;
 
+    if (fe::prepare_phase1(T, N1, p1.W) != cudaSuccess || fe::prepare_phase2(N2, p2.in) != cudaSuccess)
+        return FENGINE_ECUDA;
     // one intermediate buffer: slabs run back to back on the caller's stream
     for (long long qb = 0; qb < M; qb += SL) {
         const int qc = (int)((M - qb) < SL ? (M - qb) : SL);
         p1.q_begin = p2.q_begin = (int)qb;
         p1.q_count = p2.q_count = qc;
         p1.rows = fe::phase1_rows(T, N1, N2, qc, ns);
-        if (fe::launch_phase1(T, N1, p1, ns, st) != cudaSuccess) return FENGINE_ECUDA;
-        if (fe::launch_phase2(N2, p2, nant, st) != cudaSuccess) return FENGINE_ECUDA;
+        // the next slab's phase 1 overwrites the buffer this one's phase 2 reads: it waits as a whole
+        if (fe::launch_phase1(T, N1, p1, ns, st, qb == 0) != cudaSuccess) return FENGINE_ECUDA;
+        if (fe::launch_phase2(N2, p2, nant, st, true) != cudaSuccess) return FENGINE_ECUDA;
     }
     return FENGINE_OK;
 }
