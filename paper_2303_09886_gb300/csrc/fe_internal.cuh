@@ -97,6 +97,7 @@ struct Phase1Params {
 constexpr int kInPairs = 0;   // FP32, [stream][a_spectra / 2][k1][t2] of (re, re, im, im) of two spectra
 constexpr int kInHalf = 1;    // FP16 (re, im) pairs, [stream][a_spectra][k1][t2] (tensor-core phase 1, FP16 form)
 constexpr int kInFloat = 2;   // FP32 (re, im), [stream][a_spectra][k1][t2] (BF16 form, and N1 = 64)
+constexpr int kInHalfPairs = 3;   // FP16, as kInPairs (FP16 form, n_channels >= 16384; N2 = 1024 only)
 inline int phase1_layout(int N1) { return N1 <= 32 ? kInPairs : kInFloat; }   // what k_phase1 writes
 
 struct Phase2Params {
@@ -291,6 +292,7 @@ struct Phase1TcParams {
     int *err;                 // set to 2 if a bounded wait gave up
 };
 int phase1_tc_R(int N);
+int phase1_tc_layout(int N, int precision);   // layout of the intermediate that phase 1 writes
 bool phase1_tc_supported(int N, int T, int precision);
 int phase1_tc_phys(int N, int T, int precision);
 void build_phase1_tc_tables(int N, int T, int precision, const float *w, std::vector<uint16_t> &bmat,

@@ -135,6 +135,13 @@ __device__ __forceinline__ void mma_f16_ss(uint32_t d_tmem, uint64_t a, uint64_t
         "l"(a), "l"(b), "r"(idesc), "r"(acc));
 }
 
+// one lane of the (converged) warp
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred q;\n\telect.sync _|q, 0xFFFFFFFF;\n\tselp.u32 %0, 1, 0, q;\n\t}\n" : "=r"(p));
+    return p != 0;
+}
+
 __device__ __forceinline__ void mma_commit(uint32_t mbar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(mbar)
                  : "memory");
@@ -790,6 +797,487 @@ __global__ void __launch_bounds__(tc_threads(tc_one_cta(PH, R, T, PREC)), tc_one
     if (warp == WMMA) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEMC));
 }
 
+// ---------------------------------------------------------------------------
+// R >= 4 (n_channels >= 16384): the same contraction with the operand blocks
+// streamed. An output column then sums over R physical columns, whose operand
+// blocks (NM = 48 or 80 rows: every k1) do not fit in shared memory for a
+// useful number of columns at a time; splitting k1 instead reads every sample
+// once per slice. So the accumulators stay: a CTA takes units of CW adjacent
+// output columns x G tiles of 128 spectra, G CW NM columns of tensor memory,
+// and goes over the (c, j) operand blocks once, each used by the G tiles while
+// the next is on its way:
+//   for c, j: block B(c, j); for g: D[g][c] += A(g, c, j) B(c, j)
+// Two (c, j) steps (blocks and the G tiles' sequences) make a stage (ts_sj), loaded
+// and released as a whole (a wait, a commit and their latency per stage).
+// Units go to the CTAs round robin, so that the CTAs running at one time share
+// a few columns' operand blocks (L2) and complete each other's output sectors.
+// Roles and barriers as in k_phase1_tc; a tile whose coarse delay steps takes
+// one more round over the blocks per run. The epilogue exchanges the values of
+// two columns between the lanes of a spectrum pair and stores the second
+// stage's pairs, 16 bytes (FP16: 8) per lane.
+//
+// What bounds it: with one lane running the MMA loop, its issue (0.557 ms ->
+// 0.36 at R = 4 in FP16); since the whole warp runs it and one elected lane
+// issues, an MMA (128 x 80 x 16 at R = 8) takes 127 cycles, of which the
+// tensor core needs 40 and its shared-memory reads 52; the operand blocks come
+// from L2 at 2.2 TB/s, the sequences and results move 1.2 TB/s of HBM. Whole
+// figures: phase1_tc_streamed.
+constexpr int kTsCW = 2;
+__host__ __device__ constexpr int ts_g(int R) { return R == 8 ? 3 : 4; }
+__host__ __device__ constexpr int ts_bblk(int R, int T, int prec) {   // bytes of an operand block, all planes
+    return (prec == 2 ? 2 : 1) * tc_nm(R, 1) * 8 * tc_tp(T) * 2;
+}
+__host__ __device__ constexpr int ts_ablk(int T, int prec) { return (prec == 2 ? 2 : 1) * tc_xl(T) * 2; }
+__host__ __device__ constexpr int ts_step(int R, int T, int prec) {   // bytes of a (c, j) step: block and sequences
+    return ts_bblk(R, T, prec) + ts_g(R) * ts_ablk(T, prec);
+}
+// steps per stage: two, where two stages of two fit (all but BF16 with 32 taps)
+__host__ __device__ constexpr int ts_sj(int R, int T, int prec) {
+    return 4 * ts_step(R, T, prec) + 512 <= kTcSmemMax ? 2 : 1;
+}
+__host__ __device__ constexpr int ts_stage(int R, int T, int prec) { return ts_sj(R, T, prec) * ts_step(R, T, prec); }
+__host__ __device__ constexpr int ts_ns(int R, int T, int prec) {      // stages in flight
+    return 4 * ts_stage(R, T, prec) + 512 <= kTcSmemMax ? 4 : 3 * ts_stage(R, T, prec) + 512 <= kTcSmemMax ? 3 : 2;
+}
+__host__ __device__ constexpr int ts_smem(int R, int T, int prec) {
+    const int b = ts_ns(R, T, prec) * ts_stage(R, T, prec) + 512;
+    return b < 120 * 1024 ? 120 * 1024 : b;   // one CTA per SM (it takes the whole tensor memory)
+}
+constexpr int kTsThreads = 32 * 10, kTsFill = 128;   // 4 epilogue warps, 4 fill warps, the MMA warp, the operand warp
+
+struct TsPre {                // an item's delay flags and delays, loaded a unit ahead
+    unsigned char f[4];
+    int c_row0, c0;
+};
+struct TsTile {               // a tile and its current run [ra, rb) of delay c; ra >= rows: done
+    int st, q0, rows, ra, rb, c, c0;
+    unsigned m[4];
+};
+__device__ __forceinline__ void ts_fetch(TsPre &s, const Phase1TcParams &p, int n_tiles, int n_items, long long item) {
+    const int lane = threadIdx.x & 31;
+    if (item >= n_items) return;
+    const int st = (int)item / n_tiles, q0 = p.q_begin + ((int)item % n_tiles) * kTcRows;
+    const int rows = min(kTcRows, p.q_begin + p.q_count - q0);
+    const unsigned char *cf = p.cchg + (long long)st * p.M + q0;
+#pragma unroll
+    for (int k = 0; k < 4; k++) s.f[k] = (32 * k + lane < rows) ? __ldg(cf + 32 * k + lane) : (unsigned char)0;
+    s.c_row0 = __ldg(p.ctab + (long long)st * p.M + q0);
+    s.c0 = __ldg(p.ctab + (long long)st * p.M);
+}
+__device__ __forceinline__ void ts_run_end(TsTile &t) {   // rb: the first delay change after ra
+    int rb = t.rows;
+#pragma unroll
+    for (int k = 0; k < 4; k++) {
+        const int lo = t.ra + 1 - 32 * k;
+        unsigned mk = t.m[k];
+        if (lo >= 32) mk = 0u;
+        else if (lo > 0) mk &= ~0u << lo;
+        if (mk && rb == t.rows) rb = 32 * k + __ffs(mk) - 1;
+    }
+    t.rb = rb < t.rows ? rb : t.rows;
+}
+__device__ __forceinline__ void ts_open(TsTile &t, const TsPre &s, const Phase1TcParams &p, int n_tiles, int n_items,
+                                        long long item) {
+    const bool in = item < n_items;
+    t.st = in ? (int)item / n_tiles : 0;
+    t.q0 = p.q_begin + (in ? ((int)item % n_tiles) * kTcRows : 0);
+    t.rows = in ? min(kTcRows, p.q_begin + p.q_count - t.q0) : 0;
+#pragma unroll
+    for (int k = 0; k < 4; k++) t.m[k] = __ballot_sync(0xFFFFFFFFu, in && s.f[k] != 0);
+    t.ra = 0;
+    t.c = s.c_row0;
+    t.c0 = s.c0;
+    ts_run_end(t);
+}
+__device__ __forceinline__ void ts_next(TsTile &t, const Phase1TcParams &p) {
+    if (t.ra >= t.rows) return;
+    t.ra = t.rb;
+    if (t.ra >= t.rows) return;
+    t.c = __ldg(p.ctab + (long long)t.st * p.M + t.q0 + t.ra);
+    ts_run_end(t);
+}
+
+template <int R, int T, int PREC>
+__global__ void __launch_bounds__(kTsThreads, 1) k_phase1_ts(const __grid_constant__ Phase1TcParams p) {
+    constexpr int CW = kTsCW, G = ts_g(R), NM = tc_nm(R, 1), TP = tc_tp(T), K = 8 * TP, XL = tc_xl(T), H1 = 4 * R;
+    constexpr int NPL = PREC == 2 ? 2 : 1;                    // planes of data and operands (BF16: hi and lo)
+    constexpr int BB = ts_bblk(R, T, PREC), AB = ts_ablk(T, PREC), ST = ts_stage(R, T, PREC), NS = ts_ns(R, T, PREC);
+    constexpr int SJ = ts_sj(R, T, PREC);                     // steps per stage
+    static_assert(ts_smem(R, T, PREC) <= kTcSmemMax && NS >= 2, "two stages fit");
+    constexpr int NST = CW * R / SJ;                       // stages per round
+    constexpr int NG = (2 * (H1 + 1) + 7) / 8;                // 8-column groups holding (Re, Im) of 4 k1
+    static_assert(G * CW * NM <= 512 && G <= 4, "tensor memory; a fill warp per tile");
+    static_assert(R % SJ == 0, "a stage's steps are of one column");
+    extern __shared__ __align__(1024) uint8_t smem[];         // [NS]: blocks [SJ][BB], sequences [SJ][G][NPL][XL]
+    unsigned long long *bar = reinterpret_cast<unsigned long long *>(smem + NS * ST);
+    unsigned long long *full = bar, *empty = bar + NS, *tfull = bar + 2 * NS, *tempty = tfull + G;
+    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(tempty + G);
+    volatile int *abort_sm = reinterpret_cast<volatile int *>(tmem_slot + 1);
+
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int n_tiles = (p.q_count + kTcRows - 1) / kTcRows, n_items = p.n_streams * n_tiles;
+    const int n_ig = (n_items + G - 1) / G;
+    const int P = p.N / 8, N2 = p.N2;
+    const int n_units = (N2 / CW) * n_ig;
+    if (tid == 0) {
+        for (int i = 0; i < NS; i++) {   // full: the operand warp and a fill warp per tile
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(&full[i])), "r"(1 + G));
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&empty[i])));
+        }
+        for (int i = 0; i < G; i++) {
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&tfull[i])));
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(&tempty[i])), "r"(128));
+        }
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        *abort_sm = 0;
+    }
+    if (warp == 8) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(tmem_slot)),
+                     "r"(512));
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = *tmem_slot;
+    pdl_release();
+    pdl_wait();   // the columns and the delay table
+
+    // a bounded wait that also gives up once another role has
+    auto wait_bar = [&](unsigned long long *b, uint32_t parity) -> bool {
+        const uint32_t a = smem_addr(b);
+        const long long t0 = clock64();
+        while (!mbar_try(a, parity)) {
+            if (*abort_sm) return false;
+            if (clock64() - t0 > 2000000000LL) {
+                *abort_sm = 1;
+                atomicExch(p.err, 2);
+                return false;
+            }
+        }
+        return true;
+    };
+    auto arrive = [&](unsigned long long *b) {
+        asm volatile("{\n\t.reg .b64 st;\n\tmbarrier.arrive.shared::cta.b64 st, [%0];\n\t}" ::"r"(smem_addr(b))
+                     : "memory");
+    };
+    auto expect = [&](unsigned long long *b, uint32_t bytes) {
+        asm volatile("{\n\t.reg .b64 st;\n\tmbarrier.arrive.expect_tx.shared::cta.b64 st, [%0], %1;\n\t}" ::"r"(smem_addr(b)),
+                     "r"(bytes)
+                     : "memory");
+    };
+    auto bulk = [&](void *dst, const void *src, uint32_t bytes, unsigned long long *b) {
+        asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                         smem_addr(dst)),
+                     "l"(src), "r"(bytes), "r"(smem_addr(b))
+                     : "memory");
+    };
+
+    // every role walks the same units, rounds and tiles; the counters of the
+    // stages and of each accumulator run on across them
+    TsPre pre[G];
+    TsTile tl[G];
+#pragma unroll
+    for (int g = 0; g < G; g++) ts_fetch(pre[g], p, n_tiles, n_items, (long long)(blockIdx.x % n_ig) * G + g);
+    unsigned ns = 0, nt[G];   // stages begun, uses of each accumulator
+#pragma unroll
+    for (int g = 0; g < G; g++) nt[g] = 0;
+    const int ft = tid - 128;
+    bool ok = true;
+    for (int u = blockIdx.x; u < n_units && ok; u += gridDim.x) {
+        const int t2 = (u / n_ig) * CW;
+#pragma unroll
+        for (int g = 0; g < G; g++) ts_open(tl[g], pre[g], p, n_tiles, n_items, (long long)(u % n_ig) * G + g);
+        if (u + (int)gridDim.x < n_units) {
+#pragma unroll
+            for (int g = 0; g < G; g++)
+                ts_fetch(pre[g], p, n_tiles, n_items, (long long)((u + gridDim.x) % n_ig) * G + g);
+        }
+        for (;;) {
+            int nact = 0;          // tiles with a run in this round
+            bool moved = p.window_tap != nullptr;   // a run whose delay is not the columns' own
+#pragma unroll
+            for (int g = 0; g < G; g++) {
+                const bool act = tl[g].ra < tl[g].rows;
+                nact += act ? 1 : 0;
+                moved = moved || (act && tl[g].c != tl[g].c0);
+            }
+            if (nact == 0 || !ok) break;
+            if (warp >= 4 && warp < 8) {
+                // ---------------- fill ----------------
+                // a warp that has given up tells the others here, before any of them waits for it
+                int go = ok;
+                asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.s32 q, %1, 0;\n\tbar.red.and.pred q, 1, %2, q;\n\t"
+                             "selp.s32 %0, 1, 0, q;\n\t}\n"
+                             : "=r"(go)
+                             : "r"(go), "n"(kTsFill)
+                             : "memory");
+                ok = go != 0;
+                if (!moved) {
+                    // the columns' own delay: a sequence starts at row 8 (m0 + q0) - rb, 16-byte aligned; one
+                    // bulk copy per plane, each warp its own tile
+#pragma unroll
+                    for (int g = 0; g < G; g++) {
+                        if (warp != 4 + g || lane != 0) continue;
+                        const TsTile &ps = tl[g];
+                        const bool act = ps.ra < ps.rows;
+                        const uint16_t *col = p.cols + ((long long)ps.st * P + t2) * p.RTP + (8LL * (p.m0 + ps.q0) - p.rb);
+                        for (int k = 0; k < NST && ok; k++) {
+                            const unsigned n = ns + (unsigned)k, s = n % NS;
+                            ok = n < NS || wait_bar(&empty[s], ((n / NS) - 1) & 1);
+                            if (!ok) break;
+                            if (!act) {
+                                arrive(&full[s]);
+                                continue;
+                            }
+                            expect(&full[s], SJ * AB);
+#pragma unroll
+                            for (int i = 0; i < SJ; i++) {
+                                const int cj = k * SJ + i;
+                                const uint16_t *src = col + (long long)(cj / R + N2 * (cj % R)) * p.RTP;
+                                uint8_t *xb = smem + s * ST + SJ * BB + (i * G + g) * AB;
+#pragma unroll
+                                for (int pl = 0; pl < NPL; pl++)
+                                    bulk(xb + pl * XL * 2, src + pl * p.plane_elems, XL * 2, &full[s]);
+                            }
+                        }
+                    }
+                    __syncwarp();
+                    ok = __shfl_sync(0xFFFFFFFFu, (int)ok, 0) != 0;
+                } else {
+                    for (int k = 0; k < NST && ok; k++) {
+                        const unsigned n = ns + (unsigned)k, s = n % NS;
+                        // the decision to go on is the same in every fill thread
+                        go = ft != 0 || n < NS || wait_bar(&empty[s], ((n / NS) - 1) & 1);
+                        asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.s32 q, %1, 0;\n\tbar.red.and.pred q, 1, %2, q;\n\t"
+                                     "selp.s32 %0, 1, 0, q;\n\t}\n"
+                                     : "=r"(go)
+                                     : "r"(go), "n"(kTsFill)
+                                     : "memory");
+                        ok = go != 0;
+                        if (!ok) break;
+#pragma unroll 1
+                        for (int i = 0; i < SJ; i++) {
+                            const int c = (k * SJ + i) / R, j = (k * SJ + i) % R;
+                            const long long t = t2 + c + (long long)N2 * j;   // physical column
+#pragma unroll
+                            for (int g = 0; g < G; g++) {
+                                const TsTile &ps = tl[g];
+                                if (ps.ra >= ps.rows) continue;
+                                uint8_t *xb = smem + s * ST + SJ * BB + (i * G + g) * AB;
+                                // 16-byte chunks from the aligned element row0 - sh, each output chunk 16 bytes
+                                // at byte offset 2 sh of two consecutive source chunks
+                                const long long a0 = (long long)p.N * (p.m0 + ps.q0) - ps.c + ps.c0 + t;
+                                const long long ra = floor_div(a0, P);
+                                const long long row0 = ra - p.rb;
+                                const uint16_t *src =
+                                    p.cols + ((long long)ps.st * P + (a0 - ra * P)) * p.RTP + (row0 & ~7LL);
+                                const int sh = (int)(row0 & 7);
+                                constexpr int CPC = XL / 8;
+                                for (int e = ft; e < NPL * CPC; e += kTsFill) {
+                                    const int pl = e / CPC, q8 = e - pl * CPC;
+                                    const uint4 *q = reinterpret_cast<const uint4 *>(src + pl * p.plane_elems) + q8;
+                                    const uint4 v0 = __ldg(q), v1 = __ldg(q + 1);
+                                    const uint32_t w[8] = {v0.x, v0.y, v0.z, v0.w, v1.x, v1.y, v1.z, v1.w};
+                                    const uint32_t sel = (sh & 1) ? 0x5432u : 0x3210u;   // 2-byte shift for odd sh
+                                    uint32_t o[4];
+#pragma unroll
+                                    for (int m = 0; m < 4; m++) {
+                                        uint32_t lo = w[m], hi = w[m + 1];
+                                        if ((sh >> 1) == 1) lo = w[m + 1], hi = w[m + 2];
+                                        else if ((sh >> 1) == 2) lo = w[m + 2], hi = w[m + 3];
+                                        else if ((sh >> 1) == 3) lo = w[m + 3], hi = w[m + 4];
+                                        o[m] = __byte_perm(lo, hi, sel);
+                                    }
+                                    reinterpret_cast<uint4 *>(xb + pl * XL * 2)[q8] = make_uint4(o[0], o[1], o[2], o[3]);
+                                }
+                                if (p.window_tap) {
+                                    // debug tap: the first FIR tap of spectrum q0 + v / 8 at offset P (v % 8) + t
+                                    asm volatile("bar.sync 1, %0;" ::"n"(kTsFill) : "memory");
+                                    const uint16_t *xv = reinterpret_cast<const uint16_t *>(xb);
+                                    for (int vv = ft; vv < 8 * kTcRows; vv += kTsFill) {
+                                        const int mrow = vv >> 3;
+                                        if (mrow < ps.ra || mrow >= ps.rb) continue;
+                                        float x;
+                                        if constexpr (PREC == 2)
+                                            x = __bfloat162float(__ushort_as_bfloat16(xv[vv])) +
+                                                __bfloat162float(__ushort_as_bfloat16(xv[XL + vv]));
+                                        else x = __half2float(__ushort_as_half(xv[vv]));
+                                        p.window_tap[((long long)ps.st * p.M + ps.q0 + mrow) * p.N +
+                                                     (long long)P * (vv & 7) + t] = (int)x;
+                                    }
+                                }
+                            }
+                        }
+                        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                        asm volatile("bar.sync 1, %0;" ::"n"(kTsFill) : "memory");
+                        if (lane == 0 && warp < 4 + G) arrive(&full[s]);
+                    }
+                }
+            } else if (warp == 9) {
+                // ---------------- operand blocks ----------------
+                if (lane == 0) {
+                    for (int k = 0; k < NST && ok; k++) {
+                        const unsigned n = ns + (unsigned)k, s = n % NS;
+                        ok = n < NS || wait_bar(&empty[s], ((n / NS) - 1) & 1);
+                        if (!ok) break;
+                        expect(&full[s], SJ * BB);
+                        bulk(smem + s * ST,
+                             reinterpret_cast<const uint8_t *>(p.bmat) + ((long long)t2 * R + k * SJ) * BB, SJ * BB,
+                             &full[s]);
+                    }
+                }
+                __syncwarp();
+                ok = __shfl_sync(0xFFFFFFFFu, (int)ok, 0) != 0;
+            } else if (warp == 8) {
+                // ---------------- MMA ----------------
+                // the whole warp runs the loop (waits, addresses and descriptors stay warp-uniform, in uniform
+                // registers), one elected lane issues
+                constexpr uint32_t idesc = mma_idesc(kTcRows, NM, PREC == 2 ? 1 : 0);
+                for (int k = 0; k < NST; k++) {
+                    const unsigned n = ns + (unsigned)k, s = n % NS;
+                    ok = __all_sync(0xFFFFFFFFu, wait_bar(&full[s], (n / NS) & 1));
+                    if (!ok) break;
+                    tc_fence_after();
+                    const uint64_t bs = mat_desc(smem_addr(smem + s * ST), (NM / 8) * 128u, 128u);
+                    const uint64_t as = mat_desc(smem_addr(smem + s * ST + SJ * BB), 16u, 128u);
+                    const int c = k * SJ / R, j0 = k * SJ % R;   // (a stage's steps are of one column)
+#pragma unroll
+                    for (int g = 0; g < G; g++) {
+                        if (!ok || !__any_sync(0xFFFFFFFFu, tl[g].ra < tl[g].rows)) continue;
+                        if (k == 0 && nt[g] > 0) {   // the accumulator's last use has been read
+                            ok = __all_sync(0xFFFFFFFFu, wait_bar(&tempty[g], (nt[g] - 1) & 1));
+                            if (!ok) continue;
+                            tc_fence_after();
+                        }
+                        const uint32_t d = tmem + (uint32_t)(g * CW * NM + c * NM);
+                        if (elect_one()) {
+#pragma unroll
+                            for (int i = 0; i < SJ; i++) {
+                                // FP16: x B. BF16: x_hi B_hi + x_lo B_hi + x_hi B_lo
+#pragma unroll
+                                for (int pp = 0; pp < (PREC == 2 ? 3 : 1); pp++) {
+#pragma unroll
+                                    for (int kk = 0; kk < K / 16; kk++) {
+                                        // (start addresses in 16-byte units, in the descriptors' low bits)
+                                        const uint64_t ad =
+                                            as + (uint64_t)((i * G + g) * AB + (pp == 1 ? XL * 2 : 0) + 32 * kk) / 16;
+                                        const uint64_t bd =
+                                            bs + (uint64_t)(i * BB + (pp == 2 ? NM * K * 2 : 0) + kk * 2 * (NM / 8) * 128) / 16;
+                                        mma_f16_ss(d, ad, bd, idesc, ((j0 + i) | pp | kk) ? 1u : 0u);
+                                    }
+                                }
+                            }
+                            if (k == NST - 1) mma_commit(smem_addr(&tfull[g]));
+                        }
+                        __syncwarp();
+                    }
+                    if (!ok) break;
+                    if (elect_one()) mma_commit(smem_addr(&empty[s]));   // the stage is read
+                    __syncwarp();
+                }
+#pragma unroll
+                for (int g = 0; g < G; g++)
+                    if (tl[g].ra < tl[g].rows) nt[g]++;
+            } else {
+                // ---------------- epilogue ----------------
+                const int row = 32 * warp + lane;   // tensor-memory lane = spectrum row
+                const float osc0 = __ldg(p.oscale + t2), osc1 = __ldg(p.oscale + t2 + 1);
+#pragma unroll 1
+                for (int g = 0; g < G && ok; g++) {
+                    TsTile ps;   // tl[g] (registers: selected by comparison)
+#pragma unroll
+                    for (int i = 0; i < G; i++)
+                        if (i == g) ps = tl[i];
+                    unsigned use = 0;
+#pragma unroll
+                    for (int i = 0; i < G; i++)
+                        if (i == g) use = nt[i];
+                    if (ps.ra >= ps.rows) continue;
+                    ok = lane == 0 ? wait_bar(&tfull[g], use & 1) : true;
+                    ok = __shfl_sync(0xFFFFFFFFu, (int)ok, 0) != 0;
+                    if (!ok) break;
+                    tc_fence_after();
+                    const bool valid = row >= ps.ra && row < ps.rb;
+                    const bool both = __shfl_xor_sync(0xFFFFFFFFu, (int)valid, 1) != 0 && valid;
+                    const int odd = lane & 1;
+                    const uint32_t trow = tmem + (uint32_t)(g * CW * NM) + ((uint32_t)(32 * warp) << 16);
+                    // this pair's (k1 = 0, t2 + odd) in the second stage's pairs
+                    const long long pair = (long long)ps.st * (p.a_spectra >> 1) + ((ps.q0 + row - p.q_begin) >> 1);
+                    const long long o0 = pair * (H1 + 1) * N2 + t2;
+#pragma unroll 1
+                    for (int gq = 0; gq < NG; gq++) {
+                        float va[8], vb[8];
+                        tmem_ld8(trow + (uint32_t)(8 * gq), va);
+                        tmem_ld8(trow + (uint32_t)(NM + 8 * gq), vb);
+                        tmem_ld_wait();
+                        if (gq == NG - 1) {
+                            tc_fence_before();
+                            arrive(&tempty[g]);
+                        }
+#pragma unroll
+                        for (int kq = 0; kq < 4; kq++) {
+                            const int k1 = 4 * gq + kq;
+                            if (k1 > H1) break;
+                            const float r0 = va[2 * kq] * osc0, i0 = va[2 * kq + 1] * osc0;
+                            const float r1 = vb[2 * kq] * osc1, i1 = vb[2 * kq + 1] * osc1;
+                            // the even lane (first spectrum) finishes column t2, the odd one column t2 + 1
+                            const float rx = __shfl_xor_sync(0xFFFFFFFFu, odd ? r0 : r1, 1);
+                            const float ix = __shfl_xor_sync(0xFFFFFFFFu, odd ? i0 : i1, 1);
+                            const float ra_ = odd ? rx : r0, rb_ = odd ? r1 : rx, ia = odd ? ix : i0, ib = odd ? i1 : ix;
+                            const long long o = o0 + (long long)k1 * N2;
+                            if constexpr (PREC == 2) {
+                                float4 *A = reinterpret_cast<float4 *>(p.A) + o;
+                                if (both) {
+                                    __stcs(A + odd, make_float4(ra_, rb_, ia, ib));
+                                } else if (valid) {   // a delay step inside the pair, or its last spectrum missing
+                                    float *f = reinterpret_cast<float *>(A);
+                                    f[odd] = r0;
+                                    f[2 + odd] = i0;
+                                    f[4 + odd] = r1;
+                                    f[6 + odd] = i1;
+                                }
+                            } else {
+                                uint2 *A = reinterpret_cast<uint2 *>(p.A) + o;
+                                if (both) {
+                                    const __half2 hr = __floats2half2_rn(ra_, rb_), hi = __floats2half2_rn(ia, ib);
+                                    A[odd] = make_uint2(*reinterpret_cast<const uint32_t *>(&hr),
+                                                        *reinterpret_cast<const uint32_t *>(&hi));
+                                } else if (valid) {
+                                    __half *f = reinterpret_cast<__half *>(A);
+                                    f[odd] = __float2half_rn(r0);
+                                    f[2 + odd] = __float2half_rn(i0);
+                                    f[4 + odd] = __float2half_rn(r1);
+                                    f[6 + odd] = __float2half_rn(i1);
+                                }
+                            }
+                        }
+                    }
+                }
+#pragma unroll
+                for (int g = 0; g < G; g++)
+                    if (tl[g].ra < tl[g].rows) nt[g]++;
+            }
+            ns += NST;
+#pragma unroll
+            for (int g = 0; g < G; g++) ts_next(tl[g], p);
+        }
+    }
+    // teardown: every role has left its loop (the epilogue has read the last
+    // accumulator, so every MMA has completed; or a wait gave up: give the
+    // tensor core and the copies in flight a bounded moment to finish)
+    __syncthreads();
+    if (*abort_sm && warp == 8) {
+        const long long t0 = clock64();
+        while (clock64() - t0 < 20000000LL) {
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    if (warp == 8) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512));
+}
+
 // ---------------------------------------------------------------- host side
 
 // Physical FIR columns per CTA for an N-point transform: 16 where tc_phys
@@ -817,15 +1305,36 @@ bool phase1_tc_supported(int N, int T, int precision) {
            tc_ks(phase1_tc_phys(N, T, precision), R, T, precision) > 0;
 }
 
+// The streamed kernel takes every shape of R >= 4: per 67 M samples (16 taps)
+// phase 1 takes 0.215 ms at R = 4 and 0.231 at R = 8 in FP16, 0.364 and 0.440
+// in BF16, against 0.557, 0.846, 0.948 and 1.947 with resident operand blocks.
+bool phase1_tc_streamed(int N) { return phase1_tc_R(N) >= 4; }
+
+int phase1_tc_layout(int N, int precision) {
+    if (phase1_tc_streamed(N)) return precision == 2 ? kInPairs : kInHalfPairs;
+    return precision == 2 ? kInFloat : kInHalf;
+}
+
 void build_phase1_tc_tables(int N, int T, int precision, const float *w, std::vector<uint16_t> &bmat,
                             std::vector<float> &oscale, float &s_int) {
-    const int R = phase1_tc_R(N), P = N / 8, N2 = P / R, PH = phase1_tc_phys(N, T, precision), CW = PH / R;
-    const int KS = tc_ks(PH, R, T, precision), KPS = tc_kps(R, KS), NM = tc_nm(R, KS), TP = tc_tp(T), K = 8 * TP;
+    const bool streamed = phase1_tc_streamed(N);
+    const int R = phase1_tc_R(N), P = N / 8, N2 = P / R, PH = streamed ? R : phase1_tc_phys(N, T, precision);
+    const int CW = PH / R, KS = streamed ? 1 : tc_ks(PH, R, T, precision);
+    const int KPS = tc_kps(R, KS), NM = tc_nm(R, KS), TP = tc_tp(T), K = 8 * TP;
     const int H1 = 4 * R, NPB = precision == 2 ? 2 : 1;
     const int n_cg = N2 / CW;
-    // [column group][k1-slice][plane][physical column][NM x K]
+    // resident blocks: [column group][k1-slice][plane][physical column][NM x K];
+    // streamed (one column per group, one slice): [column][physical column][plane][NM x K]
+    const size_t plane_step = (size_t)(streamed ? 1 : PH) * NM * K, col_step = (size_t)(streamed ? NPB : 1) * NM * K;
     bmat.assign((size_t)n_cg * KS * NPB * PH * NM * K, 0);
     oscale.assign(N2, 1.0f);
+    // exp(-2 pi i ph / N), every phase the blocks use
+    std::vector<double> cs(N), sn(N);
+    for (int ph = 0; ph < N; ph++) {
+        const double ang = -2.0 * M_PI * (double)ph / (double)N;
+        cs[ph] = std::cos(ang);
+        sn[ph] = std::sin(ang);
+    }
     // global scale of the FP16 intermediate: |Z| <= 512 sum_j sum_r |w[t + P r]|
     double zmax = 0.0;
     for (int t2 = 0; t2 < N2; t2++) {
@@ -854,18 +1363,14 @@ void build_phase1_tc_tables(int N, int T, int precision, const float *w, std::ve
             for (int sl = 0; sl < KS; sl++)
                 for (int j = 0; j < R; j++) {
                     const long long t = t2 + (long long)N2 * j;
-                    const size_t blk0 = (((size_t)cgi * KS + sl) * NPB * PH + j * CW + c) * NM * K;
-                    for (int nrow = 0; nrow < NM; nrow++) {
+                    const size_t blk0 = ((size_t)cgi * KS + sl) * NPB * PH * NM * K + (size_t)(j * CW + c) * col_step;
+                    for (int nrow = 0; nrow < 2 * KPS; nrow++) {
                         const int k1 = sl * KPS + nrow / 2, im = nrow % 2;
-                        for (int k = 0; k < K; k++) {
-                            const int t1 = k % 8, jj = k / 8;
-                            double val = 0.0;
-                            if (nrow / 2 < KPS && k1 <= H1 && jj < T) {
-                                const long long tf = (long long)P * t1 + t;
-                                const long long ph = ((long long)k1 * tf) % N;
-                                const double ang = -2.0 * M_PI * (double)ph / (double)N;
-                                val = (double)w[t + (long long)P * k] * (im ? std::sin(ang) : std::cos(ang)) * sB;
-                            }
+                        if (k1 > H1) break;
+                        for (int k = 0; k < 8 * T; k++) {
+                            const long long tf = (long long)P * (k % 8) + t;
+                            const long long ph = ((long long)k1 * tf) % N;
+                            const double val = (double)w[t + (long long)P * k] * (im ? sn[ph] : cs[ph]) * sB;
                             const size_t off =
                                 (size_t)(k / 8) * (NM / 8) * 64 + (nrow / 8) * 64 + (nrow % 8) * 8 + (k % 8);
                             if (precision == 2) {
@@ -873,7 +1378,7 @@ void build_phase1_tc_tables(int N, int T, int precision, const float *w, std::ve
                                 const __nv_bfloat16 hi = __float2bfloat16_rn((float)val);
                                 const __nv_bfloat16 lo = __float2bfloat16_rn((float)(val - (double)__bfloat162float(hi)));
                                 bmat[blk0 + off] = __bfloat16_as_ushort(hi);
-                                bmat[blk0 + (size_t)PH * NM * K + off] = __bfloat16_as_ushort(lo);
+                                bmat[blk0 + plane_step + off] = __bfloat16_as_ushort(lo);
                             } else {
                                 bmat[blk0 + off] = __half_as_ushort(__float2half_rn((float)val));
                             }
@@ -914,16 +1419,44 @@ static cudaError_t launch_tc(const Phase1TcParams &p, cudaStream_t s, bool pdl) 
     }
 }
 
+template <int R, int T, int PREC>
+static cudaError_t launch_ts(const Phase1TcParams &p, cudaStream_t s, bool pdl) {
+    constexpr int smem = ts_smem(R, T, PREC);
+    if constexpr (smem > kTcSmemMax) {
+        return cudaErrorInvalidValue;   // refused when the plan is made
+    } else {
+        cudaError_t e =
+            cudaFuncSetAttribute(k_phase1_ts<R, T, PREC>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e != cudaSuccess) return e;
+        const long long tiles = (p.q_count + kTcRows - 1) / kTcRows, ig = (p.n_streams * tiles + ts_g(R) - 1) / ts_g(R);
+        const long long units = (long long)(p.N2 / kTsCW) * ig;
+        const int grid = (int)(units < p.splits ? units : p.splits);
+        return launch_kernel(k_phase1_ts<R, T, PREC>, dim3((unsigned)grid), (unsigned)kTsThreads, (size_t)smem, s, pdl, p);
+    }
+}
+
 template <int R, int PREC>
 static cudaError_t launch_tc_t(int T, const Phase1TcParams &p, cudaStream_t s, bool pdl) {
-    switch (T) {
-        case 1: return launch_tc<R, 1, PREC>(p, s, pdl);
-        case 2: return launch_tc<R, 2, PREC>(p, s, pdl);
-        case 4: return launch_tc<R, 4, PREC>(p, s, pdl);
-        case 8: return launch_tc<R, 8, PREC>(p, s, pdl);
-        case 16: return launch_tc<R, 16, PREC>(p, s, pdl);
-        case 32: return launch_tc<R, 32, PREC>(p, s, pdl);
-        default: return cudaErrorInvalidValue;
+    if constexpr (R >= 4) {
+        switch (T) {
+            case 1: return launch_ts<R, 1, PREC>(p, s, pdl);
+            case 2: return launch_ts<R, 2, PREC>(p, s, pdl);
+            case 4: return launch_ts<R, 4, PREC>(p, s, pdl);
+            case 8: return launch_ts<R, 8, PREC>(p, s, pdl);
+            case 16: return launch_ts<R, 16, PREC>(p, s, pdl);
+            case 32: return launch_ts<R, 32, PREC>(p, s, pdl);
+            default: return cudaErrorInvalidValue;
+        }
+    } else {
+        switch (T) {
+            case 1: return launch_tc<R, 1, PREC>(p, s, pdl);
+            case 2: return launch_tc<R, 2, PREC>(p, s, pdl);
+            case 4: return launch_tc<R, 4, PREC>(p, s, pdl);
+            case 8: return launch_tc<R, 8, PREC>(p, s, pdl);
+            case 16: return launch_tc<R, 16, PREC>(p, s, pdl);
+            case 32: return launch_tc<R, 32, PREC>(p, s, pdl);
+            default: return cudaErrorInvalidValue;
+        }
     }
 }
 

@@ -213,6 +213,7 @@ static cudaError_t launch_p2_in(int in, const GroupArgs<Phase2Params, CAP> *g, c
     switch (in) {
         case kInPairs: return launch_p2<N2, kInPairs, CAP>(g, s, pdl);
         case kInHalf: return launch_p2<N2, kInHalf, CAP>(g, s, pdl);
+        case kInHalfPairs: return cudaErrorInvalidValue;   // N2 = 1024 only
         default: return launch_p2<N2, kInFloat, CAP>(g, s, pdl);
     }
 }

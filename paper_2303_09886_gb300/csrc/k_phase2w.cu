@@ -116,6 +116,7 @@ __device__ __forceinline__ float4 as_float4(cpair c) { return make_float4(c.x.x,
 // antennas.
 template <int IN, int CAP>
 __global__ void __launch_bounds__(kWThreads, 1) k_phase2w(const __grid_constant__ GroupArgs<Phase2Params, CAP> ga) {
+    constexpr bool kPaired = IN == kInPairs || IN == kInHalfPairs, kHalf = IN == kInHalf || IN == kInHalfPairs;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     WSmem &sm = *reinterpret_cast<WSmem *>(smem_raw);
     const int mem = CAP == 1 ? 0 : group_member(ga, (int)blockIdx.x);
@@ -178,20 +179,20 @@ __global__ void __launch_bounds__(kWThreads, 1) k_phase2w(const __grid_constant_
     // intermediate holds an even number of spectra, so that a pair's second one is there even past the last.
     auto pair_at = [&](const WItem &w) -> long long {
         const long long row = (long long)(w.ant * 2 + pol) * p.a_spectra + (w.q0 - p.q_begin) + 2 * pr;
-        return ((IN == kInPairs ? row >> 1 : row) * (H1 + 1) + w.k1) * kWN2;
+        return ((kPaired ? row >> 1 : row) * (H1 + 1) + w.k1) * kWN2;
     };
     auto active_in = [&](const WItem &w) { return w.q0 + 2 * pr < p.q_begin + p.q_count; };
-    // into its buffer (one lane): one run of 16 KB where phase 1 wrote pairs, else the two sequences behind
+    // into its buffer (one lane): one run where phase 1 wrote pairs, else the two sequences behind
     // each other
     auto fetch = [&](const WItem &w) {
         constexpr uint32_t EB = IN == kInPairs ? 16 : IN == kInHalf ? 4 : 8;
-        constexpr uint32_t bytes = (IN == kInPairs ? 1u : 2u) * EB * kWN2;
+        constexpr uint32_t bytes = (kPaired ? 1u : 2u) * EB * kWN2;
         asm volatile("{\n\t.reg .b64 st;\n\tmbarrier.arrive.expect_tx.shared::cta.b64 st, [%0], %1;\n\t}" ::"r"(mbar),
                      "r"(bytes)
                      : "memory");
         const char *a = reinterpret_cast<const char *>(p.A) + pair_at(w) * EB;
         bulk_copy(sm_addr(tile), a, EB * kWN2, mbar);
-        if constexpr (IN != kInPairs)
+        if constexpr (!kPaired)
             bulk_copy(sm_addr(tile) + EB * kWN2, a + (long long)(H1 + 1) * kWN2 * EB, EB * kWN2, mbar);
     };
     // (delta, phi / pi) of the warp's two spectra, and their gain sets (set 0 without timed gains)
@@ -269,7 +270,7 @@ __global__ void __launch_bounds__(kWThreads, 1) k_phase2w(const __grid_constant_
             {
                 const float inv = 2.0f / (float)N;
                 // P carries the inverse of the FP16 intermediate's scale (a power of two)
-                const float u = IN == kInHalf ? p.tc_unscale : 1.0f;
+                const float u = kHalf ? p.tc_unscale : 1.0f;
                 float s0, c0, s1, c1;
                 sincospif(f0.y - f0.x * (float)(k1 + N1 * lane) * inv, &s0, &c0);
                 sincospif(f1.y - f1.x * (float)(k1 + N1 * lane) * inv, &s1, &c1);
@@ -304,6 +305,14 @@ __global__ void __launch_bounds__(kWThreads, 1) k_phase2w(const __grid_constant_
                 if constexpr (IN == kInPairs) {
 #pragma unroll
                     for (int a = 0; a < 32; a++) z[a] = as_cpair(lin[32 * a + lane]);
+                } else if constexpr (IN == kInHalfPairs) {
+                    const uint2 *hp2 = reinterpret_cast<const uint2 *>(lin);
+#pragma unroll
+                    for (int a = 0; a < 32; a++) {
+                        const uint2 v = hp2[32 * a + lane];
+                        z[a] = cpair{__half22float2(*reinterpret_cast<const __half2 *>(&v.x)),
+                                     __half22float2(*reinterpret_cast<const __half2 *>(&v.y))};
+                    }
                 } else if constexpr (IN == kInHalf) {
                     const __half2 *hb = reinterpret_cast<const __half2 *>(lin);
 #pragma unroll
@@ -474,6 +483,7 @@ static cudaError_t launch_w_in(int in, const GroupArgs<Phase2Params, CAP> *g, cu
     switch (in) {
         case kInPairs: return launch_w<kInPairs, CAP>(g, s, pdl);
         case kInHalf: return launch_w<kInHalf, CAP>(g, s, pdl);
+        case kInHalfPairs: return launch_w<kInHalfPairs, CAP>(g, s, pdl);
         default: return launch_w<kInFloat, CAP>(g, s, pdl);
     }
 }
