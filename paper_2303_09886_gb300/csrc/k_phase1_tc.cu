@@ -550,9 +550,14 @@ __global__ void __launch_bounds__(tc_threads(tc_one_cta(PH, R, T, PREC)), tc_one
                          : "memory");
             if (!ok) break;
             uint16_t *xb = xsm + (size_t)s * NPL * PH * XL;
-            if (!p.window_tap && ps.c == ps.c0) {
-                // the pass's delay is the columns' c0: every column sequence starts at
-                // row 8 (m0 + q0) - rb, 16-byte aligned, one bulk copy each (per plane)
+            // the columns are laid out at delay c0: a pass at delay c reads column
+            // t + c0 - c, which for all but the CTAs at the edges is one of the same
+            // rows: only those realign (32768 channels in BF16, 2^28 samples at a
+            // delay rate of 5e-9, whose delay steps once or twice: a call 8.50 -> 4.77 ms)
+            const int dc = ps.c0 - ps.c;
+            if (!p.window_tap && dc + cg * CW >= 0 && dc + (cg + 1) * CW <= N2) {
+                // every column sequence starts at row 8 (m0 + q0) - rb, 16-byte
+                // aligned, one bulk copy each (per plane)
                 if (ft == 0) {
                     constexpr uint32_t bytes = (uint32_t)(NPL * PH * XL * 2);
                     asm volatile("{\n\t.reg .b64 st;\n\tmbarrier.arrive.expect_tx.shared::cta.b64 st, [%0], %1;\n\t}"
@@ -561,7 +566,7 @@ __global__ void __launch_bounds__(tc_threads(tc_one_cta(PH, R, T, PREC)), tc_one
 #pragma unroll 1
                     for (int i = 0; i < NPL * PH; i++) {
                         const int ic = i % PH, pl = i / PH;
-                        const long long t = (long long)cg * CW + (ic % CW) + (long long)N2 * (ic / CW);
+                        const long long t = (long long)cg * CW + dc + (ic % CW) + (long long)N2 * (ic / CW);
                         const uint16_t *src = p.cols + pl * p.plane_elems + ((long long)ps.st * P + t) * p.RTP + row0;
                         asm volatile(
                             "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
@@ -998,12 +1003,14 @@ __global__ void __launch_bounds__(kTsThreads, 1) k_phase1_ts(const __grid_consta
         }
         for (;;) {
             int nact = 0;          // tiles with a run in this round
-            bool moved = p.window_tap != nullptr;   // a run whose delay is not the columns' own
+            bool moved = p.window_tap != nullptr;   // a run that reads other rows than the columns' own delay
 #pragma unroll
             for (int g = 0; g < G; g++) {
                 const bool act = tl[g].ra < tl[g].rows;
                 nact += act ? 1 : 0;
-                moved = moved || (act && tl[g].c != tl[g].c0);
+                // a run at another delay reads other columns of the same rows, where none of the unit's wraps
+                const int dc = tl[g].c0 - tl[g].c;
+                moved = moved || (act && (dc + t2 < 0 || dc + t2 + CW > N2));
             }
             if (nact == 0 || !ok) break;
             if (warp >= 4 && warp < 8) {
@@ -1017,14 +1024,15 @@ __global__ void __launch_bounds__(kTsThreads, 1) k_phase1_ts(const __grid_consta
                              : "memory");
                 ok = go != 0;
                 if (!moved) {
-                    // the columns' own delay: a sequence starts at row 8 (m0 + q0) - rb, 16-byte aligned; one
-                    // bulk copy per plane, each warp its own tile
+                    // a sequence starts at row 8 (m0 + q0) - rb, 16-byte aligned, of column t + c0 - c (the
+                    // columns are laid out at delay c0); one bulk copy per plane, each warp its own tile
 #pragma unroll
                     for (int g = 0; g < G; g++) {
                         if (warp != 4 + g || lane != 0) continue;
                         const TsTile &ps = tl[g];
                         const bool act = ps.ra < ps.rows;
-                        const uint16_t *col = p.cols + ((long long)ps.st * P + t2) * p.RTP + (8LL * (p.m0 + ps.q0) - p.rb);
+                        const uint16_t *col =
+                            p.cols + ((long long)ps.st * P + t2 + (ps.c0 - ps.c)) * p.RTP + (8LL * (p.m0 + ps.q0) - p.rb);
                         for (int k = 0; k < NST && ok; k++) {
                             const unsigned n = ns + (unsigned)k, s = n % NS;
                             ok = n < NS || wait_bar(&empty[s], ((n / NS) - 1) & 1);
