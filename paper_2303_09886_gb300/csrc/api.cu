@@ -320,7 +320,7 @@ fengine_status fengine_plan_create(const fengine_config *cfg, fengine_plan_t *ou
     const int ns = pl->n_streams;
     cudaError_t e = cudaSuccess;
     if ((!tc1 && (e = fe::prepare_phase1(T, N1, pl->W)) != cudaSuccess) ||
-        (e = fe::prepare_phase2(pl->N2, tc1 ? fe::phase1_tc_layout((int)N, cfg->precision) : fe::phase1_layout(N1))) != cudaSuccess) {
+        (e = fe::prepare_phase2(pl->N2, tc1 ? fe::phase1_tc_layout((int)N, cfg->precision) : fe::kInPairs)) != cudaSuccess) {
         release(pl);
         return cuda_fail(e, "kernel attributes");
     }
@@ -748,7 +748,7 @@ fengine_status process_impl(fengine_plan_t pl, void *cuda_stream, const uint8_t 
     p2.out = d_out;
     p2.prequant = reinterpret_cast<float2 *>(d_prequant);
     p2.a_spectra = pl->SL;
-    p2.in = pl->tc1 ? fe::phase1_tc_layout(pl->N, pl->precision) : fe::phase1_layout(pl->N1);
+    p2.in = pl->tc1 ? fe::phase1_tc_layout(pl->N, pl->precision) : fe::kInPairs;
     p2.err = pl->d_err;
     p2.tc_unscale = pl->tc_unscale;
 

@@ -242,7 +242,7 @@ fengine_status fengine_batch_process(fengine_batch_t b, void *cuda_stream, const
                     total += blocks;
                 }
                 g2.start[nm] = total;
-                if (fe::launch_phase2_group(N2, fe::phase1_layout(N1), g2, gs) != cudaSuccess) return FENGINE_ECUDA;
+                if (fe::launch_phase2_group(N2, fe::kInPairs, g2, gs) != cudaSuccess) return FENGINE_ECUDA;
             }
         }
     }

@@ -80,68 +80,12 @@ __host__ __device__ constexpr float cos64(int q) {
     return c[q];
 }
 
-// a * exp(-2 pi i Q / 64) for a compile-time Q in [0, 32]: Q = 0 and
-// Q = 16 (-i) fold to moves; otherwise cos - i sin with sin(2 pi Q / 64) =
-// cos(2 pi |16 - Q| / 64).
-template <int Q>
-__device__ __forceinline__ float2 cmul_w64(float2 a) {
-    static_assert(Q >= 0 && Q <= 32, "twiddle index");
-    if constexpr (Q == 0) {
-        return a;
-    } else if constexpr (Q == 16) {
-        return make_float2(a.y, -a.x);
-    } else {
-        constexpr float c = cos64(Q), s = cos64(Q <= 16 ? 16 - Q : Q - 16);
-        return cmul(a, make_float2(c, -s));
-    }
-}
-
-namespace detail {
-
-// bins 1 .. NN/4 - 1 of the real DFT from the half-length DFTs E and O
-template <int NN, int K>
-__device__ __forceinline__ void rdit_combine(float2 (&X)[NN / 2 + 1], const float2 (&E)[NN / 4 + 1],
-                                             const float2 (&O)[NN / 4 + 1]) {
-    if constexpr (K < NN / 4) {
-        const float2 t = cmul_w64<K * (64 / NN)>(O[K]);
-        X[K] = cadd2(E[K], t);
-        const float2 d = csub2(E[K], t);
-        X[NN / 2 - K] = make_float2(d.x, -d.y);
-        rdit_combine<NN, K + 1>(X, E, O);
-    }
-}
-
-}  // namespace detail
-
-// In-register real DFT of NN points (NN = 2, 4, ..., 64): bins 0..NN/2 of
-// X[k] = sum_t x[t] exp(-2 pi i k t / NN), radix-2 decimation in time on the
-// real sequence. With E and O the half-length DFTs of the even and odd
-// samples (both real sequences, so E[NN/2 - k] = conj E[k]),
+// The in-register transforms are radix-2 decimations in time with every index
+// and twiddle a compile-time constant. A real DFT of NN points (bins 0..NN/2 of
+// X[k] = sum_t x[t] exp(-2 pi i k t / NN)) takes the half-length DFTs E and O of
+// the even and odd samples (both real sequences, so E[NN/2 - k] = conj E[k]):
 //   X[k] = E[k] + w^k O[k],  X[NN/2 - k] = conj(E[k] - w^k O[k]),  k <= NN/4,
-// w = exp(-2 pi i / NN); w^(NN/4) = -i and the k = 0 terms are real. Every
-// index and twiddle is a compile-time constant.
-template <int NN>
-__device__ __forceinline__ void rdft_reg(const float (&x)[NN], float2 (&X)[NN / 2 + 1]) {
-    if constexpr (NN == 2) {
-        X[0] = make_float2(x[0] + x[1], 0.0f);
-        X[1] = make_float2(x[0] - x[1], 0.0f);
-    } else {
-        constexpr int H = NN / 2, Q = NN / 4;
-        float xe[H], xo[H];
-#pragma unroll
-        for (int t = 0; t < H; t++) {
-            xe[t] = x[2 * t];
-            xo[t] = x[2 * t + 1];
-        }
-        float2 E[Q + 1], O[Q + 1];
-        rdft_reg<H>(xe, E);
-        rdft_reg<H>(xo, O);
-        X[0] = make_float2(E[0].x + O[0].x, 0.0f);
-        X[H] = make_float2(E[0].x - O[0].x, 0.0f);
-        detail::rdit_combine<NN, 1>(X, E, O);
-        X[Q] = make_float2(E[Q].x, -O[Q].x);
-    }
-}
+// w = exp(-2 pi i / NN); w^(NN/4) = -i and the k = 0 terms are real.
 
 // ---- two sequences at a time ----
 //
@@ -178,13 +122,6 @@ __device__ __forceinline__ cpair cmulp(cpair a, cpair b) {
     if constexpr (IMB) r.y = __ffma2_rn(a.y, b.x, __fmul2_rn(a.x, b.y));
     else r.y = __ffma2_rn(a.x, b.y, __fmul2_rn(a.y, b.x));
     return r;
-}
-
-// cmulp for one sequence
-template <bool IMB>
-__device__ __forceinline__ float2 cmul_rn(float2 a, float2 b) {
-    return make_float2(__fmaf_rn(a.x, b.x, -__fmul_rn(a.y, b.y)),
-                       IMB ? __fmaf_rn(a.y, b.x, __fmul_rn(a.x, b.y)) : __fmaf_rn(a.x, b.y, __fmul_rn(a.y, b.x)));
 }
 
 // a * exp(-2 pi i Q / 64) for a compile-time Q (not 0 or 16): signs go with the
@@ -241,7 +178,7 @@ __device__ __forceinline__ void rdit_combine2(cpair (&X)[NN / 2 + 1], const cpai
 
 }  // namespace detail
 
-// rdft_reg of two real sequences (x[t]: sample t of both).
+// Real DFTs of two sequences (x[t]: sample t of both), NN = 2, 4, ..., 32.
 template <int NN>
 __device__ __forceinline__ void rdft_reg2(const float2 (&x)[NN], cpair (&X)[NN / 2 + 1]) {
     if constexpr (NN == 2) {
@@ -283,59 +220,6 @@ __device__ __forceinline__ void fft_regc2(cpair (&z)[NN]) {
         fft_regc2<NN / 2>(e);
         fft_regc2<NN / 2>(o);
         detail::dit_combine2<NN, 0>(z, e, o);
-    }
-}
-
-// fft_regc2 whose two halves change places where s = (-1, -1): z[K] and
-// z[K + NN / 2] hold X[K] and X[K + NN / 2] for s = (1, 1), and X[K + NN / 2]
-// and X[K] for s = (-1, -1) (the last sums as fused products by s, exact), so
-// that two warps can keep different halves of a transform in the same registers.
-template <int NN, int K>
-__device__ __forceinline__ void dit_combine2_half(cpair (&z)[NN], const cpair (&e)[NN / 2], const cpair (&o)[NN / 2],
-                                                  float2 s, float2 m) {
-    if constexpr (K < NN / 2) {
-        constexpr int Q = K * (64 / NN);
-        cpair t = o[K];
-        if constexpr (Q == 16) {   // times -i: t = (o.y, -o.x)
-            z[K].x = __ffma2_rn(t.y, s, e[K].x);
-            z[K].y = __ffma2_rn(t.x, m, e[K].y);
-            z[K + NN / 2].x = __ffma2_rn(t.y, m, e[K].x);
-            z[K + NN / 2].y = __ffma2_rn(t.x, s, e[K].y);
-        } else {
-            if constexpr (Q != 0) t = cmulp_w64<Q, Q < 16 && Q != 8>(o[K]);
-            z[K].x = __ffma2_rn(t.x, s, e[K].x);
-            z[K].y = __ffma2_rn(t.y, s, e[K].y);
-            z[K + NN / 2].x = __ffma2_rn(t.x, m, e[K].x);
-            z[K + NN / 2].y = __ffma2_rn(t.y, m, e[K].y);
-        }
-        dit_combine2_half<NN, K + 1>(z, e, o, s, m);
-    }
-}
-template <int NN>
-__device__ __forceinline__ void fft_regc2_half(cpair (&z)[NN], float2 s, float2 m) {   // m = -s
-    cpair e[NN / 2], o[NN / 2];
-#pragma unroll
-    for (int t = 0; t < NN / 2; t++) {
-        e[t] = z[2 * t];
-        o[t] = z[2 * t + 1];
-    }
-    fft_regc2<NN / 2>(e);
-    fft_regc2<NN / 2>(o);
-    dit_combine2_half<NN, 0>(z, e, o, s, m);
-}
-
-// z[K] times exp(-2 pi i K / 32), K = K0 .. K1 - 1 (the second half of a
-// 32-point transform from its odd points), element K in z[K - K0 + Z0]
-template <int K, int K1, int Z>
-__device__ __forceinline__ void twiddle32(cpair (&z)[16]) {
-    if constexpr (K < K1) {
-        if constexpr (K == 8) {   // -i
-            const cpair t = z[Z];
-            z[Z] = cpair{t.y, neg2(t.x)};
-        } else if constexpr (K != 0) {
-            z[Z] = cmulp_w64<2 * K, (K < 8 && K != 4)>(z[Z]);
-        }
-        twiddle32<K + 1, K1, Z + 1>(z);
     }
 }
 

@@ -96,9 +96,8 @@ struct Phase1Params {
 // Layouts of the intermediate between the phases (a_spectra is even):
 constexpr int kInPairs = 0;   // FP32, [stream][a_spectra / 2][k1][t2] of (re, re, im, im) of two spectra
 constexpr int kInHalf = 1;    // FP16 (re, im) pairs, [stream][a_spectra][k1][t2] (tensor-core phase 1, FP16 form)
-constexpr int kInFloat = 2;   // FP32 (re, im), [stream][a_spectra][k1][t2] (BF16 form, and N1 = 64)
+constexpr int kInFloat = 2;   // FP32 (re, im), [stream][a_spectra][k1][t2] (BF16 form below 16384 channels)
 constexpr int kInHalfPairs = 3;   // FP16, as kInPairs (FP16 form, n_channels >= 16384; N2 = 1024 only)
-inline int phase1_layout(int N1) { return N1 <= 32 ? kInPairs : kInFloat; }   // what k_phase1 writes
 
 struct Phase2Params {
     const float2 *A;          // the intermediate in the layout `in`, spectrum q at row q - q_begin

@@ -26,8 +26,10 @@
 // to shared memory as pairs of output rows, and for each (row pair, t2) the
 // real N1-point DFT over t1 of both rows runs in packed registers, is
 // multiplied by the twiddle and stored as the second stage reads it: the two
-// spectra of a pair side by side, (re, re, im, im). N1 = 64 keeps one row per
-// thread (the pair would not fit in registers) and stores FP32 (re, im).
+// spectra of a pair side by side, (re, re, im, im). For N1 = 64 two threads
+// share the transform (the pair would not fit in one's registers): 1024
+// spectra of 32768 channels, 16 taps: 0.385 ms and 0.234 in the second stage,
+// against 0.40 and 0.25 with one row per thread and spectra stored apart.
 //
 // What bounds it: the FP32 pipe (a packed instruction takes two of its
 // cycles; 43 % active) and the dependent chains of 16 warps per SM, the
@@ -55,9 +57,10 @@ struct P1Shape {
     static constexpr int CW = C < 64 ? C : 64;      // columns of one warp
     static constexpr int NW = C / CW;        // warps that filter
     static constexpr int NS = CW / W;        // segments (t1 values) of one warp
-    static constexpr bool PAIR = N1 <= 32;   // row pairs through the DFT and in the output
-    static constexpr int GROW = PAIR ? 2 * C : C + 8;   // floats per row pair (PAIR) or row of g
-    static constexpr int G_FLOATS = PAIR ? (kP1Block / 2) * GROW : kP1Block * GROW;
+    // floats per row pair of g (N1 = 64: a warp of the DFT reads 4 row pairs at a time, half a warp on
+    // 32 banks)
+    static constexpr int GROW = 2 * C + (N1 == 64 ? 16 : 0);
+    static constexpr int G_FLOATS = (kP1Block / 2) * GROW;
     // Staged input: the packed bytes of each (input row, t1 segment of W
     // columns) are copied into the ring from the segment's first byte rounded
     // down to ALIGN, SEG bytes (the W samples' bytes plus up to 15 in front
@@ -70,7 +73,7 @@ struct P1Shape {
     static constexpr unsigned ALIGN = C == 32 ? 8u : 16u;   // rows of N = 32 samples are 40 bytes apart
     static constexpr int ROWB = NS * SEG;    // staged bytes per row of one warp
     static constexpr int STAGE_BYTES = NW * RING * ROWB + 16;   // (a row's last 32-bit word may reach past it)
-    static constexpr int TW_FLOATS = (N1 / 2 + 1) * W * (PAIR ? 4 : 2);
+    static constexpr int TW_FLOATS = (N1 / 2 + 1) * W * 4;
     // T = 32 goes over a block in two sweeps of 16 taps, the second adding to g (the weights and the
     // window of 32 taps would not fit in registers; the sums are the two halves of T = 32 as it is)
     static constexpr int TT = T > 16 ? 16 : T;
@@ -147,17 +150,30 @@ struct P1Stage {
 #pragma unroll
         for (int k = 0; k < PER; k++) {
             const int e = lane + 32 * k, row = e / CPR;
-            if ((S::SG * CPR % 32 == 0 || e < S::SG * CPR) && row >= row_lo && row < rows_left) {
-                if (fast) {
-                    p1_cp_async16(dst + 16u * (unsigned)e, chunk0 + V[k]);
-                } else {
+            const bool in = (S::SG * CPR % 32 == 0 || e < S::SG * CPR) && row >= row_lo && row < rows_left;
+            if (fast) {
+                if (in) p1_cp_async16(dst + 16u * (unsigned)e, chunk0 + V[k]);
+            } else if constexpr (N1 == 64) {
+                // word by word, the four words of a copy on adjacent lanes: segments of 32 bytes would have an
+                // instruction's words on 32 lines (16 taps, 36 spectra of 32768 channels, whose first rows lie in
+                // the history: 0.058 -> 0.033 ms; with the longer segments of N1 <= 32 the plain order is the faster)
 #pragma unroll
-                    for (int i = 0; i < 4; i++) {
-                        const unsigned v = V[k] + 4u * (unsigned)i;   // below 0 wraps past total
+                for (int i = 0; i < 4; i++) {
+                    const int el = 8 * i + (lane >> 2), e4 = el + 32 * k, row4 = e4 / CPR;
+                    const unsigned v = __shfl_sync(0xFFFFFFFFu, V[k], el) + 4u * (unsigned)(lane & 3);   // below 0 wraps past total
+                    if ((S::SG * CPR % 32 == 0 || e4 < S::SG * CPR) && row4 >= row_lo && row4 < rows_left) {
                         const bool ok = v < total;
                         const uint8_t *src = ok && v >= hb ? chunk0 + v : hist + (ok ? v : 0u);
-                        p1_cp_async4(dst + 16u * (unsigned)e + 4u * (unsigned)i, src, ok ? 4u : 0u);
+                        p1_cp_async4(dst + 16u * (unsigned)e4 + 4u * (unsigned)(lane & 3), src, ok ? 4u : 0u);
                     }
+                }
+            } else if (in) {
+#pragma unroll
+                for (int i = 0; i < 4; i++) {
+                    const unsigned v = V[k] + 4u * (unsigned)i;   // below 0 wraps past total
+                    const bool ok = v < total;
+                    const uint8_t *src = ok && v >= hb ? chunk0 + v : hist + (ok ? v : 0u);
+                    p1_cp_async4(dst + 16u * (unsigned)e + 4u * (unsigned)i, src, ok ? 4u : 0u);
                 }
             }
             V[k] += RB * (unsigned)S::SG;
@@ -213,7 +229,7 @@ __device__ __forceinline__ float sample10_at(const uint8_t *hist, const uint8_t 
 // adjacent: two floats on in a row, or four in a row pair).
 template <class S>
 __device__ __forceinline__ int p1_gpos(int r, int c) {
-    return S::PAIR ? (r >> 1) * S::GROW + 2 * c + (r & 1) : r * S::GROW + c;
+    return (r >> 1) * S::GROW + 2 * c + (r & 1);
 }
 
 // Output rows (r, r + 1) of a column pair from the ring win of TT + 1 input
@@ -237,29 +253,16 @@ __device__ __forceinline__ void p1_fir_pair(int r, const float2 (&win)[S::TT + 1
         b0 = __ffma2_rn(w2[j], win[(r + j) % (T + 1)], b0);
         b1 = __ffma2_rn(w2[j], win[(r + 1 + j) % (T + 1)], b1);
     }
-    if constexpr (S::PAIR) {
-        float4 o = make_float4(a0.x, a1.x, a0.y, a1.y);
-        float4 *g = reinterpret_cast<float4 *>(g0 + (r >> 1) * S::GROW);
-        if constexpr (TH < T) {   // scalar sums, straight into the order of the row pair
-            o = make_float4(__fadd_rn(a0.x, b0.x), __fadd_rn(a1.x, b1.x), __fadd_rn(a0.y, b0.y),
-                            __fadd_rn(a1.y, b1.y));
-        } else if (S::SWEEPS > 1 && add) {
-            const float4 u = *g;
-            o = make_float4(__fadd_rn(u.x, o.x), __fadd_rn(u.y, o.y), __fadd_rn(u.z, o.z), __fadd_rn(u.w, o.w));
-        }
-        *g = o;
-    } else {
-        float2 *ga = reinterpret_cast<float2 *>(g0 + r * S::GROW), *gb = reinterpret_cast<float2 *>(g0 + (r + 1) * S::GROW);
-        if constexpr (TH < T) {
-            a0 = __fadd2_rn(a0, b0);
-            a1 = __fadd2_rn(a1, b1);
-        } else if (S::SWEEPS > 1 && add) {
-            a0 = __fadd2_rn(*ga, a0);
-            a1 = __fadd2_rn(*gb, a1);
-        }
-        *ga = a0;
-        *gb = a1;
+    float4 o = make_float4(a0.x, a1.x, a0.y, a1.y);
+    float4 *g = reinterpret_cast<float4 *>(g0 + (r >> 1) * S::GROW);
+    if constexpr (TH < T) {   // scalar sums, straight into the order of the row pair
+        o = make_float4(__fadd_rn(a0.x, b0.x), __fadd_rn(a1.x, b1.x), __fadd_rn(a0.y, b0.y),
+                        __fadd_rn(a1.y, b1.y));
+    } else if (S::SWEEPS > 1 && add) {
+        const float4 u = *g;
+        o = make_float4(__fadd_rn(u.x, o.x), __fadd_rn(u.y, o.y), __fadd_rn(u.z, o.z), __fadd_rn(u.w, o.w));
     }
+    *g = o;
 }
 
 // General case of the FIR: a run of output rows [ra, rb) of a block with a
@@ -311,14 +314,108 @@ __device__ __noinline__ void p1_fir_general(const Phase1Params &p, const uint8_t
     }
 }
 
+// X[k1] of a row pair times its twiddle, into the intermediate.
+template <int N1, int K1>
+__device__ __forceinline__ void p1_store(const cpair &X, const float4 *tp, float4 *out, long long N2, int W) {
+    const float4 t = tp[K1 * W];   // (re, re, im, im)
+    const cpair tc{make_float2(t.x, t.y), make_float2(t.z, t.w)};
+    cpair b;
+    if constexpr (K1 == 0 || K1 == N1 / 2) {   // real
+        b.x = __fmul2_rn(X.x, tc.x);
+        b.y = __fmul2_rn(X.x, tc.y);
+    } else {
+        b = cmulp<(K1 < N1 / 4)>(X, tc);
+    }
+    __stcs(out + K1 * N2, make_float4(b.x.x, b.x.y, b.y.x, b.y.y));
+}
+template <int N1, int W, int K1, int KE>
+__device__ __forceinline__ void p1_store_all(const cpair (&X)[N1 / 2 + 1], const float4 *tp, float4 *out, long long N2) {
+    if constexpr (K1 <= KE) {
+        p1_store<N1, K1>(X[K1], tp, out, N2, W);
+        p1_store_all<N1, W, K1 + 1, KE>(X, tp, out, N2);
+    }
+}
+
+// Bins K .. KE (<= 15) and 32 - K of the 64-point real DFT from the 32-point ones of the even and odd
+// samples (rdit_combine2), stored.
+template <int W, int K, int KE>
+__device__ __forceinline__ void p1_combine64(const cpair *E, const cpair *O, const float4 *tp, float4 *out, long long N2) {
+    if constexpr (K <= KE) {
+        const cpair t = cmulp_w64<K, (K < 8)>(O[K]), e = E[K];
+        cpair X;
+        X.x = __fadd2_rn(e.x, t.x);
+        X.y = __fadd2_rn(e.y, t.y);
+        p1_store<64, K>(X, tp, out, N2, W);
+        X.x = sub2(e.x, t.x);
+        X.y = sub2(t.y, e.y);
+        p1_store<64, 32 - K>(X, tp, out, N2, W);
+        p1_combine64<W, K + 1, KE>(E, O, tp, out, N2);
+    }
+}
+
+// Half of a 64-point real DFT of a row pair: one thread transforms the even samples (H = 0), one in
+// another warp the odd ones; they exchange the bins that the other finishes through the slots of g that
+// each has read (own: slot of its first sample), and finish K = 0 .. 8 and 9 .. 16 (bins K and 32 - K).
+template <int W, int H>
+__device__ __forceinline__ void p1_half64(float2 *g, bool act, int bar, const float4 *tp, float4 *out, long long N2) {
+    // (a thread without a pair goes along up to its stores: its slots are its own, and their values unused)
+    cpair Z[17];
+    {
+        float2 x[32];
+#pragma unroll
+        for (int i = 0; i < 32; i++) x[i] = g[(2 * i + H) * W];
+        rdft_reg2<32>(x, Z);
+    }
+    constexpr int S0 = H ? 0 : 9;
+#pragma unroll
+    for (int i = 0; i < (H ? 9 : 8); i++) {
+        g[(4 * i + H) * W] = Z[S0 + i].x;
+        if (S0 + i != 0 && S0 + i != 16) g[(4 * i + 2 + H) * W] = Z[S0 + i].y;
+    }
+    asm volatile("bar.sync %0, 64;" ::"r"(bar) : "memory");
+    if (!act) return;
+    constexpr int K0 = H ? 9 : 0, R = 1 - H;
+    cpair Y[17];   // the other half's
+#pragma unroll
+    for (int i = 0; i < (H ? 8 : 9); i++) {
+        Y[K0 + i].x = g[(4 * i + R) * W];
+        if (K0 + i != 0 && K0 + i != 16) Y[K0 + i].y = g[(4 * i + 2 + R) * W];
+    }
+    cpair X;
+    if constexpr (H == 0) {
+        X.x = __fadd2_rn(Z[0].x, Y[0].x);
+        p1_store<64, 0>(X, tp, out, N2, W);
+        X.x = sub2(Z[0].x, Y[0].x);
+        p1_store<64, 32>(X, tp, out, N2, W);
+        p1_combine64<W, 1, 8>(Z, Y, tp, out, N2);
+    } else {
+        p1_combine64<W, 9, 15>(Y, Z, tp, out, N2);
+        X.x = Y[16].x;
+        X.y = neg2(Z[16].x);
+        p1_store<64, 16>(X, tp, out, N2, W);
+    }
+}
+
 // The real N1-point DFT over t1 of the rows of a block in g, the twiddle and
 // the store of B[k1][t2]. qa: the block's first row in the intermediate.
 template <int N1, int W, class S>
-__device__ __forceinline__ void p1_dft(const Phase1Params &p, const float *g, const float *tw, int rows, int stream,
-                                       int qa, int t2_0) {
+__device__ __forceinline__ void p1_dft(const Phase1Params &p, float *g, const float *tw, int rows, int stream, int qa,
+                                       int t2_0) {
     constexpr int H1 = N1 / 2;
     const int N2 = p.N2;
-    if constexpr (S::PAIR) {
+    const long long pair0 = (long long)stream * (p.a_spectra >> 1) + (qa >> 1);
+    if constexpr (N1 == 64) {
+        // two warps per 32 (row pair, t2): a thread with both halves would need 256 registers
+        static_assert((kP1Block / 2) * W * 2 == kP1Threads, "one pass");
+        const int wq = (threadIdx.x >> 5) & 3, e = 32 * wq + (threadIdx.x & 31), rp = e / W, w = e % W;
+        const int n = ((rows + 1) >> 1) * W;
+        if (32 * wq >= n) return;
+        float2 *gp = reinterpret_cast<float2 *>(g + rp * S::GROW) + w;
+        float4 *out = reinterpret_cast<float4 *>(p.A) + (pair0 + rp) * (H1 + 1) * N2 + t2_0 + w;
+        const float4 *tp = reinterpret_cast<const float4 *>(tw) + w;
+        if (threadIdx.x < kP1Threads / 2) p1_half64<W, 0>(gp, e < n, 1 + wq, tp, out, N2);
+        else p1_half64<W, 1>(gp, e < n, 1 + wq, tp, out, N2);
+    } else {
 #pragma unroll 1
         for (int e = threadIdx.x; e < ((rows + 1) >> 1) * W; e += kP1Threads) {
             const int rp = e / W, w = e % W;
@@ -328,41 +425,8 @@ __device__ __forceinline__ void p1_dft(const Phase1Params &p, const float *g, co
             for (int t1 = 0; t1 < N1; t1++) x[t1] = gp[t1 * W];
             cpair X[H1 + 1];
             rdft_reg2<N1>(x, X);
-            float4 *out = reinterpret_cast<float4 *>(p.A) +
-                          ((long long)stream * (p.a_spectra >> 1) + (qa >> 1) + rp) * (H1 + 1) * N2 + t2_0 + w;
-            const float4 *tp = reinterpret_cast<const float4 *>(tw) + w;
-#pragma unroll
-            for (int k = 0; k <= H1; k++) {
-                const float4 t = tp[k * W];   // (re, re, im, im)
-                const cpair tc{make_float2(t.x, t.y), make_float2(t.z, t.w)};
-                cpair b;
-                if (k == 0 || k == H1) {   // real
-                    b.x = __fmul2_rn(X[k].x, tc.x);
-                    b.y = __fmul2_rn(X[k].x, tc.y);
-                } else {
-                    b = k < N1 / 4 ? cmulp<true>(X[k], tc) : cmulp<false>(X[k], tc);
-                }
-                __stcs(out + (long long)k * N2, make_float4(b.x.x, b.x.y, b.y.x, b.y.y));
-            }
-        }
-    } else {
-#pragma unroll 1
-        for (int e = threadIdx.x; e < rows * W; e += kP1Threads) {
-            const int r = e / W, w = e % W;
-            const float *gp = g + r * S::GROW + w;
-            float x[N1];
-#pragma unroll
-            for (int t1 = 0; t1 < N1; t1++) x[t1] = gp[t1 * W];
-            float2 X[H1 + 1];
-            rdft_reg<N1>(x, X);
-            float2 *out = p.A + ((long long)stream * p.a_spectra + qa + r) * (H1 + 1) * N2 + t2_0 + w;
-            const float2 *tp = reinterpret_cast<const float2 *>(tw) + w;
-            const float2 t0 = tp[0], th = tp[H1 * W];
-            out[0] = make_float2(X[0].x * t0.x, X[0].x * t0.y);
-#pragma unroll
-            for (int k = 1; k < H1; k++)
-                out[(long long)k * N2] = k < N1 / 4 ? cmul_rn<true>(X[k], tp[k * W]) : cmul_rn<false>(X[k], tp[k * W]);
-            out[(long long)H1 * N2] = make_float2(X[H1].x * th.x, X[H1].x * th.y);
+            p1_store_all<N1, W, 0, H1>(X, reinterpret_cast<const float4 *>(tw) + w,
+                                       reinterpret_cast<float4 *>(p.A) + (pair0 + rp) * (H1 + 1) * N2 + t2_0 + w, N2);
         }
     }
 }
@@ -395,8 +459,7 @@ __global__ void __launch_bounds__(kP1Threads, 2) k_phase1(const __grid_constant_
     // this tile's twiddles exp(-2 pi i k1 t2 / N) (read after the first block's barrier)
     for (int i = threadIdx.x; i < (N1 / 2 + 1) * W; i += kP1Threads) {
         const float2 v = __ldg(p.tw1 + (long long)(i / W) * N2 + t2_0 + i % W);
-        if constexpr (S::PAIR) reinterpret_cast<float4 *>(tw)[i] = make_float4(v.x, v.x, v.y, v.y);
-        else reinterpret_cast<float2 *>(tw)[i] = v;
+        reinterpret_cast<float4 *>(tw)[i] = make_float4(v.x, v.x, v.y, v.y);
     }
     pdl_release();
     pdl_wait();
@@ -473,9 +536,9 @@ __global__ void __launch_bounds__(kP1Threads, 2) k_phase1(const __grid_constant_
             return p1_fields(my + (v % S::RING) * S::ROWB, sel, sh);
         };
         // the span's first copies, of the sweep from tap j0 on
-        auto begin = [&](int j0) {
+        auto begin = [&](int j0, int n) {
             __syncwarp();   // the ring's slots of the span or sweep before have been read
-            st.start(rel_b + (unsigned)N * (unsigned)j0, N2, warp, n_out + S::TT - 1);
+            st.start(rel_b + (unsigned)N * (unsigned)j0, N2, warp, n + S::TT - 1);
             constexpr int FIRST = S::AHEAD + (S::CARRY ? S::PRE / S::SG : 0);
 #pragma unroll
             for (int gi = 0; gi < FIRST; gi++) st.group(gi * S::SG, gi == 0);
@@ -484,12 +547,12 @@ __global__ void __launch_bounds__(kP1Threads, 2) k_phase1(const __grid_constant_
                 __syncwarp();
             }
         };
-        if (fwarp && S::SWEEPS == 1) begin(0);
+        if (fwarp && S::CARRY) begin(0, n_out);
         for (; b < be; b++) {
             const int rows = min(kP1Block, Rv - b * kP1Block);
 #pragma unroll 1
             for (int j0 = 0; j0 < T; j0 += S::TT) {
-                if (fwarp && S::SWEEPS > 1) begin(j0);
+                if (fwarp && !S::CARRY) begin(j0, rows);
                 // the columns' weights, read again for every block: over a DFT stage they would take 2 T of the
                 // registers that it needs
                 float2 w2[S::TT];
@@ -529,7 +592,7 @@ __global__ void __launch_bounds__(kP1Threads, 2) k_phase1(const __grid_constant_
                             win[row % (S::TT + 1)] = p1_decode(row_at(v));
                             const int r = gi * S::SG + i - 1;   // the pair (r, r + 1) has its rows r .. r + T
                             if ((i & 1) && (S::C >= 64 || filt))
-                                p1_fir_pair<S>(r, win, w2, gs + (S::PAIR ? 2 * c : c), j0 > 0);
+                                p1_fir_pair<S>(r, win, w2, gs + 2 * c, j0 > 0);
                         }
                     }
                 }

@@ -228,7 +228,7 @@ fengine_status fengine_process_chunk_noalloc(const fengine_noalloc_args *a, cons
     p2.R2 = fe::phase2_R2(N2);
     p2.out = d_out;
     p2.prequant = nullptr;
-    p2.in = fe::phase1_layout(N1);
+    p2.in = fe::kInPairs;
     p2.a_spectra = (int)SL;
 
     if (fe::prepare_phase1(T, N1, p1.W) != cudaSuccess || fe::prepare_phase2(N2, p2.in) != cudaSuccess)

@@ -59,3 +59,16 @@ def test_gain_sets_change_inside_a_work_item():
     compare_call(s, a[0], M_, S_, n, T, delays, gains)
     b, _, _ = run_gpu(s, n, T, L, 1, delays, gains, D=32, taps=False, prequant=False)
     np.testing.assert_array_equal(a[0]["out"], b[0]["out"])
+
+
+@pytest.mark.parametrize("n,T,M,off", [(1024, 16, 33, 0), (4096, 8, 9, 4), (2048, 32, 70, 0), (8192, 4, 2, 12)])
+def test_shared_64_point_transforms(n, T, M, off):
+    """First radix 64 (two threads per transform) behind every second stage, with one to many row pairs per
+    block, windows that begin in the history, and chunks that are not 16-byte aligned (copies word by word)."""
+    L = 2 * n * M
+    s = streams(synth.SEED_BASE + 31 * n + M, 1, 2 * L, 30.0, tones=[(0.31, 60.0, 0.4)])
+    gains = [[synth.random_gains(3 * n + p, 1, n)[0] for p in range(2)]]
+    delays = [[[Seg(delay=20.2 + 5.5 * p, rate=1e-6, phase=0.4)] for p in range(2)]]
+    res, M_, S_ = run_gpu(s, n, T, L, 2, delays, gains, D=64, taps=False, fft_n1=64, in_offset=off)
+    for r in res:
+        compare_call(s, r, M_, S_, n, T, delays, gains)
