@@ -139,6 +139,13 @@ __device__ __forceinline__ cpair cmulp_w64(cpair a) {
     return r;
 }
 
+// A load of what an earlier kernel of the call wrote (programmatic launches: after pdl_wait()). Not __ldg, whose
+// loads a compiler may move above the wait, as loads of memory that nothing writes while the kernel runs.
+template <class V>
+__device__ __forceinline__ V ld_dep(const V *p) {
+    return *p;
+}
+
 namespace detail {
 
 template <int NN, int K>

@@ -470,7 +470,7 @@ __global__ void __launch_bounds__(kP1Threads, 2) k_phase1(const __grid_constant_
 #pragma unroll
     for (int b = 0; b < kP1Blocks; b++) {
         const int r = b * kP1Block + lane;
-        cdl[b] = r < Rv ? __ldg(p.ctab + (long long)stream * p.M + q0 + r) : 0;
+        cdl[b] = r < Rv ? ld_dep(p.ctab + (long long)stream * p.M + q0 + r) : 0;
     }
 
     // this thread's FIR columns (c, c + 1)

@@ -239,9 +239,9 @@ __device__ __forceinline__ void pass_prefetch(PassIter &s, const Phase1TcParams 
     const int rows = min(kTcRows, p.q_begin + p.q_count - q0);
     const unsigned char *cf = p.cchg + (long long)st * p.M + q0;
 #pragma unroll
-    for (int k = 0; k < 4; k++) s.f[k] = (32 * k + lane < rows) ? __ldg(cf + 32 * k + lane) : (unsigned char)0;
-    s.pc_row0 = __ldg(p.ctab + (long long)st * p.M + q0);
-    s.pc0 = __ldg(p.ctab + (long long)st * p.M);
+    for (int k = 0; k < 4; k++) s.f[k] = (32 * k + lane < rows) ? ld_dep(cf + 32 * k + lane) : (unsigned char)0;
+    s.pc_row0 = ld_dep(p.ctab + (long long)st * p.M + q0);
+    s.pc0 = ld_dep(p.ctab + (long long)st * p.M);
 }
 
 __device__ __forceinline__ bool warp_next_pass(PassIter &s, Pass &ps, const Phase1TcParams &p, int n_tiles) {
@@ -274,7 +274,7 @@ __device__ __forceinline__ bool warp_next_pass(PassIter &s, Pass &ps, const Phas
             if (mk && rb == s.rows) rb = 32 * k + __ffs(mk) - 1;
         }
         if (rb > s.rows) rb = s.rows;
-        const int c = s.ra == 0 ? s.c_row0 : __ldg(p.ctab + (long long)s.st * p.M + s.q0 + s.ra);
+        const int c = s.ra == 0 ? s.c_row0 : ld_dep(p.ctab + (long long)s.st * p.M + s.q0 + s.ra);
         ps = Pass{s.st, s.q0, s.ra, rb, c, s.c0};
         s.ra = rb;
         return true;
@@ -595,8 +595,8 @@ __global__ void __launch_bounds__(tc_threads(tc_one_cta(PH, R, T, PREC)), tc_one
                         const int ip = e / CPC, j = e - ip * CPC, i = ip % PH;
                         const uint4 *src =
                             reinterpret_cast<const uint4 *>(p.cols + (ip / PH) * p.plane_elems + fsrc[s * PH + i]) + j;
-                        a[u] = __ldg(src);
-                        b[u] = __ldg(src + 1);
+                        a[u] = ld_dep(src);
+                        b[u] = ld_dep(src + 1);
                     }
                 }
 #pragma unroll
@@ -868,9 +868,9 @@ __device__ __forceinline__ void ts_fetch(TsPre &s, const Phase1TcParams &p, int 
     const int rows = min(kTcRows, p.q_begin + p.q_count - q0);
     const unsigned char *cf = p.cchg + (long long)st * p.M + q0;
 #pragma unroll
-    for (int k = 0; k < 4; k++) s.f[k] = (32 * k + lane < rows) ? __ldg(cf + 32 * k + lane) : (unsigned char)0;
-    s.c_row0 = __ldg(p.ctab + (long long)st * p.M + q0);
-    s.c0 = __ldg(p.ctab + (long long)st * p.M);
+    for (int k = 0; k < 4; k++) s.f[k] = (32 * k + lane < rows) ? ld_dep(cf + 32 * k + lane) : (unsigned char)0;
+    s.c_row0 = ld_dep(p.ctab + (long long)st * p.M + q0);
+    s.c0 = ld_dep(p.ctab + (long long)st * p.M);
 }
 __device__ __forceinline__ void ts_run_end(TsTile &t) {   // rb: the first delay change after ra
     int rb = t.rows;
@@ -901,7 +901,7 @@ __device__ __forceinline__ void ts_next(TsTile &t, const Phase1TcParams &p) {
     if (t.ra >= t.rows) return;
     t.ra = t.rb;
     if (t.ra >= t.rows) return;
-    t.c = __ldg(p.ctab + (long long)t.st * p.M + t.q0 + t.ra);
+    t.c = ld_dep(p.ctab + (long long)t.st * p.M + t.q0 + t.ra);
     ts_run_end(t);
 }
 
@@ -1088,7 +1088,7 @@ __global__ void __launch_bounds__(kTsThreads, 1) k_phase1_ts(const __grid_consta
                                 for (int e = ft; e < NPL * CPC; e += kTsFill) {
                                     const int pl = e / CPC, q8 = e - pl * CPC;
                                     const uint4 *q = reinterpret_cast<const uint4 *>(src + pl * p.plane_elems) + q8;
-                                    const uint4 v0 = __ldg(q), v1 = __ldg(q + 1);
+                                    const uint4 v0 = ld_dep(q), v1 = ld_dep(q + 1);
                                     const uint32_t w[8] = {v0.x, v0.y, v0.z, v0.w, v1.x, v1.y, v1.z, v1.w};
                                     const uint32_t sel = (sh & 1) ? 0x5432u : 0x3210u;   // 2-byte shift for odd sh
                                     uint32_t o[4];

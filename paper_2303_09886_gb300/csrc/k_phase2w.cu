@@ -201,9 +201,9 @@ __global__ void __launch_bounds__(kWThreads, 1) k_phase2w(const __grid_constant_
     auto model = [&](const WItem &w) {
         const long long sq = (long long)(w.ant * 2 + pol) * M;
         const int q = w.q0 + 2 * pr, q1 = min(q + 1, p.q_begin + p.q_count - 1);
-        f0 = __ldg(p.ftab + sq + q);
-        f1 = __ldg(p.ftab + sq + q1);
-        if (p.gsel) gsel = (int)__ldg(p.gsel + sq + q) | (int)__ldg(p.gsel + sq + q1) << 8;
+        f0 = ld_dep(p.ftab + sq + q);
+        f1 = ld_dep(p.ftab + sq + q1);
+        if (p.gsel) gsel = (int)ld_dep(p.gsel + sq + q) | (int)ld_dep(p.gsel + sq + q1) << 8;
     };
     for (int e = threadIdx.x; e < 32 * 32; e += kWThreads) {
         const float2 t = __ldg(p.tw2 + (((e >> 5) * (e & 31)) & (kWN2 - 1)));
@@ -227,12 +227,12 @@ __global__ void __launch_bounds__(kWThreads, 1) k_phase2w(const __grid_constant_
         int gs0 = 0, gs1 = 0;
         if (p.gsel) {
             const unsigned char *g0 = p.gsel + (long long)(ant * 2) * M, *g1 = g0 + M;
-            gs0 = __ldg(g0 + ws.q0);
-            gs1 = __ldg(g1 + ws.q0);
+            gs0 = ld_dep(g0 + ws.q0);
+            gs1 = ld_dep(g1 + ws.q0);
             __syncthreads();
             for (int i = seg + 1 + threadIdx.x; i < class_end; i += kWThreads) {
                 const int q = ws.q0 + (i - seg) * kWR;
-                if (__ldg(g0 + q) != gs0 || __ldg(g1 + q) != gs1) {
+                if (ld_dep(g0 + q) != gs0 || ld_dep(g1 + q) != gs1) {
                     atomicMin(&sm.seg_end, i);
                     break;
                 }
