@@ -124,6 +124,16 @@ __device__ __forceinline__ cpair cmulp(cpair a, cpair b) {
     return r;
 }
 
+// a conj(b): real part fma(a.x, b.x, a.y b.y), imaginary part fma(a.y, b.x, -(a.x b.y))
+__device__ __forceinline__ cpair cmulp_conj(cpair a, cpair b) {
+    cpair r;
+    r.x = __ffma2_rn(a.x, b.x, __fmul2_rn(a.y, b.y));
+    r.y = __ffma2_rn(a.y, b.x, __fmul2_rn(neg2(a.x), b.y));
+    return r;
+}
+__device__ __forceinline__ cpair as_cpair(float4 v) { return cpair{make_float2(v.x, v.y), make_float2(v.z, v.w)}; }
+__device__ __forceinline__ float4 as_float4(cpair c) { return make_float4(c.x.x, c.x.y, c.y.x, c.y.y); }
+
 // a * exp(-2 pi i Q / 64) for a compile-time Q (not 0 or 16): signs go with the
 // variable factors, where they are free, so that the constants are the seven
 // cosines in (0, 1) and stay in registers

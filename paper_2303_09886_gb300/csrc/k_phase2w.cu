@@ -98,16 +98,6 @@ struct WSmem {
     int seg_end;
 };
 
-// a conj(b): real part fma(a.x, b.x, a.y b.y), imaginary part fma(a.y, b.x, -(a.x b.y))
-__device__ __forceinline__ cpair cmulp_conj(cpair a, cpair b) {
-    cpair r;
-    r.x = __ffma2_rn(a.x, b.x, __fmul2_rn(a.y, b.y));
-    r.y = __ffma2_rn(a.y, b.x, __fmul2_rn(neg2(a.x), b.y));
-    return r;
-}
-__device__ __forceinline__ cpair as_cpair(float4 v) { return cpair{make_float2(v.x, v.y), make_float2(v.z, v.w)}; }
-__device__ __forceinline__ float4 as_float4(cpair c) { return make_float4(c.x.x, c.x.y, c.y.x, c.y.y); }
-
 }  // namespace
 
 // Persistent: one CTA per SM (a thread holds 32 points of two spectra: 128
