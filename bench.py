@@ -242,10 +242,10 @@ def _base_streams(seed: int, n: int, sigma: float = 32.0):
 
 
 def _batched_launches(plans):
-    """Kernel launches of one fengine_batch_process over FP32 plans: one for
-    the delay table, lost-data flags and history tail per member, then per group of members with the same
-    (taps, N1, N2), one phase-1 and one phase-2 grid per slab round (at most
-    64 members per grid)."""
+    """Kernel launches of one fengine_batch_process over FP32 plans: one grid
+    for the members' delay tables, lost-data flags and history tails, then per
+    group of members with the same (taps, N1, N2) one phase-1 and one phase-2
+    grid per slab round (at most 64 members per grid)."""
     groups = {}
     for p in plans:
         groups.setdefault((p.n_taps, p.info.fft_n1, p.info.fft_n2), []).append(int(p.info.slabs_per_chunk))
@@ -254,7 +254,7 @@ def _batched_launches(plans):
         for r in range(max(slabs)):
             k = sum(1 for s in slabs if s > r)
             grids += 2 * ((k + 63) // 64)
-    return len(plans) + grids
+    return (len(plans) + 63) // 64 + grids
 
 
 def run_batched(args):

@@ -710,9 +710,13 @@ fengine_status process_impl(fengine_plan_t pl, void *cuda_stream, const uint8_t 
     pp.tail_bytes = pl->hist_bytes;
     pp.chunk_bytes = pl->chunk_bytes;
     pp.n_streams = pl->n_streams;
-    prof_begin(pl, 0, st);
-    if ((e = fe::launch_prologue(pp, st)) != cudaSuccess) return cuda_fail(e, "prologue launch");
-    prof_end(pl, st);
+    if (def) {
+        def->pro = pp;
+    } else {
+        prof_begin(pl, 0, st);
+        if ((e = fe::launch_prologue(pp, st)) != cudaSuccess) return cuda_fail(e, "prologue launch");
+        prof_end(pl, st);
+    }
 
     fe::Phase1Params p1{};
     p1.chunk = d_packed;

@@ -153,7 +153,7 @@ struct PrologueParams {
     uint8_t *hist_out;                // [stream][tail_bytes]: the last bytes of [hist_in | chunk]
     long long tail_bytes, chunk_bytes;
     int n_streams;
-    int b_delay, b_lost, b_tail;      // blocks of each part (launch_prologue sets them)
+    int b_delay, b_lost, b_tail;      // blocks of each part (the launch sets them)
 };
 cudaError_t launch_prologue(const PrologueParams &p, cudaStream_t s);
 
@@ -184,11 +184,16 @@ struct GroupArgs {
 };
 using Phase1Group = GroupArgs<Phase1Params, kMaxGroup>;
 using Phase2Group = GroupArgs<Phase2Params, kMaxGroup>;
+using PrologueGroup = GroupArgs<PrologueParams, kMaxGroup>;
+static_assert(sizeof(Phase1Group) <= 32 * 1024 - 256 && sizeof(Phase2Group) <= 32 * 1024 - 256 &&
+                  sizeof(PrologueGroup) <= 32 * 1024 - 256,
+              "a kernel's parameters");
 // one member's blocks and their (gx, gy) in its own launch
 int phase1_blocks(int N1, const Phase1Params &p, int n_streams, int *gx, int *gy);
 int phase2_blocks(int N2, const Phase2Params &p, int n_ant, int *gx, int *gy);   // N2 < 1024
 long long phase2w_items(const Phase2Params &p, int n_ant);                        // work items of k_phase2w
 int phase2w_wave();                                                                 // CTAs of one k_phase2w wave
+cudaError_t launch_prologue_group(PrologueGroup &g, cudaStream_t s);   // (fills in the members' blocks)
 cudaError_t launch_phase1_group(int T, int N1, const Phase1Group &g, cudaStream_t s);
 cudaError_t launch_phase2_group(int N2, int in, const Phase2Group &g, cudaStream_t s);
 // second stage for N2 = 1024 (launch_phase2 and launch_phase2_group route it there)
@@ -196,18 +201,19 @@ cudaError_t launch_phase2w(const Phase2Params &p, int n_ant, cudaStream_t s, boo
 cudaError_t prepare_phase2w(int in);
 cudaError_t launch_phase2w_group(int in, const Phase2Group &g, cudaStream_t s);
 
-// A call of a plan with its phase launches handed back instead of enqueued
-// (batching): the per-slab parameters fengine_process_chunk would launch.
-// The FP32 form only; its other kernels (delay table, lost data, history
-// tail) are enqueued on the call's stream as usual.
+// A call of a plan with its launches handed back instead of enqueued
+// (batching): the parameters of the prologue and of the per-slab phases that
+// fengine_process_chunk would launch. The FP32 form only; its uploads are
+// enqueued on the call's stream as usual.
 struct DeferredCall {
+    PrologueParams pro;
     int T = 0, N1 = 0, N2 = 0, n_streams = 0, n_ant = 0;
     std::vector<Phase1Params> p1;   // per slab, in order
     std::vector<Phase2Params> p2;
 };
-// whether process_chunk_deferred hands back this plan's phase launches
+// whether process_chunk_deferred hands back this plan's launches
 bool plan_defers(fengine_plan_t pl);
-// fengine_process_chunk with the FP32 form's phase launches returned in def
+// fengine_process_chunk with the FP32 form's launches returned in def
 // (*deferred = true); other forms run as fengine_process_chunk (*deferred =
 // false). No debug outputs.
 fengine_status process_chunk_deferred(fengine_plan_t pl, cudaStream_t st, const uint8_t *d_packed,

@@ -192,9 +192,13 @@ __device__ __forceinline__ void lost_block(const LostDataParams &p, const DelayT
     }
 }
 
-__global__ void __launch_bounds__(256) k_prologue(const __grid_constant__ PrologueParams p) {
+// One call's (CAP = 1) or those of a batch's members in one grid.
+template <int CAP>
+__global__ void __launch_bounds__(256) k_prologue(const __grid_constant__ GroupArgs<PrologueParams, CAP> ga) {
     pdl_release();
-    const int b = (int)blockIdx.x;
+    const int m = CAP == 1 ? 0 : group_member(ga, (int)blockIdx.x);
+    const PrologueParams &p = ga.p[m];
+    const int b = (int)blockIdx.x - (CAP == 1 ? 0 : ga.start[m]);
     if (b < p.b_delay) {
         delay_entry(p.d, (long long)b * 256 + threadIdx.x);
     } else if (b < p.b_delay + p.b_lost) {
@@ -211,13 +215,29 @@ static int tail_blocks(long long tail_bytes, int n_streams) {
     return (int)(want < 1 ? 1 : want > per ? (per < 608 ? per : 608) : want > 608 ? 608 : want);
 }
 
-cudaError_t launch_prologue(const PrologueParams &q, cudaStream_t s) {
-    PrologueParams p = q;
-    p.b_delay = (int)(((long long)p.d.n_streams * p.d.M + 255) / 256);
-    p.b_lost = p.lost ? p.l.n_ant * ((p.l.M + p.l.S - 1) / p.l.S) + 1 : 0;
-    p.b_tail = p.tail_bytes > 0 ? tail_blocks(p.tail_bytes, p.n_streams) : 0;
-    return launch_kernel(k_prologue, dim3((unsigned)(p.b_delay + p.b_lost + p.b_tail)), 256u, 0, s, false, p);
+template <int CAP>
+static cudaError_t launch_prologue_n(GroupArgs<PrologueParams, CAP> &g, cudaStream_t s) {
+    int total = 0;
+    for (int m = 0; m < g.n; m++) {
+        PrologueParams &p = g.p[m];
+        p.b_delay = (int)(((long long)p.d.n_streams * p.d.M + 255) / 256);
+        p.b_lost = p.lost ? p.l.n_ant * ((p.l.M + p.l.S - 1) / p.l.S) + 1 : 0;
+        p.b_tail = p.tail_bytes > 0 ? tail_blocks(p.tail_bytes, p.n_streams) : 0;
+        g.start[m] = total;
+        total += p.b_delay + p.b_lost + p.b_tail;
+    }
+    g.start[g.n] = total;
+    return total ? launch_kernel(k_prologue<CAP>, dim3((unsigned)total), 256u, 0, s, false, g) : cudaSuccess;
 }
+
+cudaError_t launch_prologue(const PrologueParams &p, cudaStream_t s) {
+    GroupArgs<PrologueParams, 1> g;
+    g.p[0] = p;
+    g.n = 1;
+    return launch_prologue_n(g, s);
+}
+
+cudaError_t launch_prologue_group(PrologueGroup &g, cudaStream_t s) { return launch_prologue_n(g, s); }
 
 // The history tail by itself (the down-converter's).
 __global__ void __launch_bounds__(256) k_tail_update(const uint8_t *hist_in, const uint8_t *chunk, uint8_t *hist_out,
