@@ -1,6 +1,7 @@
 // Host side of libfengine: plan state, argument checking and the launch
 // sequence of one fengine_process_chunk call. See include/fengine.h for the
 // contract of every entry point.
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
@@ -330,8 +331,9 @@ fengine_status fengine_plan_create(const fengine_config *cfg, fengine_plan_t *ou
     // buffer and one launch pair. Neither phase is bound by memory (the second
     // stage takes the same time per spectrum from L2), so smaller slabs only
     // add launches and tails: 8192 channels, 4 antennas x 2 x 2^25 samples
-    // take 0.89 ms as one slab and 1.02 ms as five of 256 MiB. Where the
-    // device has no room for it, down to the 256 MiB slab.
+    // take 0.89 ms as one slab and 1.02 ms as five of 256 MiB. Of the
+    // device's free memory a slab takes 1/32 at most, so that many plans fit
+    // side by side; the least is the 256 MiB slab.
     // intermediate element: FP32 (re, im), or FP16 (re, im) in the FP16 form
     pl->a_elem = pl->precision == FENGINE_TC_FP16 ? 4 : 8;
     const size_t per_spec = (size_t)ns * (pl->N1 / 2 + 1) * pl->N2 * pl->a_elem;
@@ -342,7 +344,10 @@ fengine_status fengine_plan_create(const fengine_config *cfg, fengine_plan_t *ou
         return s > M32 ? M32 : s;
     };
     const long long SL_min = slab_of((size_t)256 << 20);
-    long long SL = cfg->slab_spectra ? (cfg->slab_spectra > M32 ? M32 : cfg->slab_spectra) : slab_of((size_t)3 << 30);
+    size_t mem_free = 0, mem_total = 0;
+    if (cudaMemGetInfo(&mem_free, &mem_total) != cudaSuccess) mem_free = 0;
+    const long long SL_max = std::max(SL_min, slab_of(std::min((size_t)3 << 30, mem_free / 32)));
+    long long SL = cfg->slab_spectra ? (cfg->slab_spectra > M32 ? M32 : cfg->slab_spectra) : SL_max;
     size_t a_bytes = 0;
     for (;;) {
         a_bytes = (size_t)((M + SL - 1) / SL > 1 ? 2 : 1) * SL * per_spec;
