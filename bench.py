@@ -48,11 +48,11 @@ KERNEL_SOURCES = {
 }
 _CAPTURED = 33554432   # input samples of the captured launch
 NCU_TRAFFIC = {
-    "k_phase1<16,16,32,0>": {"bytes_per_sample": (44702720 + 92542720) / _CAPTURED, "src": "17209441f63721c1"},
-    "k_phase2w": {"bytes_per_sample": (170189312 + 22351616) / _CAPTURED, "src": "0ed9442a5b4bd850"},
-    "k_phase2w<half>": {"bytes_per_sample": (94110976 + 22121728) / _CAPTURED, "src": "0ed9442a5b4bd850"},
-    "k_phase1_tc<2,16,1>": {"bytes_per_sample": (96520704 + 48678144) / _CAPTURED, "src": "ea5cae1109eb0be7"},
-    "k_unpack_cols": {"bytes_per_sample": (42592512 + 19993088) / _CAPTURED, "src": "ea5cae1109eb0be7"},
+    "k_phase1<16,16,32,0>": {"bytes_per_sample": (44091392 + 90493184) / _CAPTURED, "src": "58685870f5a492cb"},
+    "k_phase2w": {"bytes_per_sample": (161295360 + 16910336) / _CAPTURED, "src": "d0c296192441a53f"},
+    "k_phase2w<half>": {"bytes_per_sample": (84109824 + 12113152) / _CAPTURED, "src": "d0c296192441a53f"},
+    "k_phase1_tc<2,16,1>": {"bytes_per_sample": (95922944 + 48432128) / _CAPTURED, "src": "581b89670166b1b5"},
+    "k_unpack_cols": {"bytes_per_sample": (42587904 + 19447296) / _CAPTURED, "src": "581b89670166b1b5"},
 }
 
 
