@@ -130,20 +130,23 @@ __device__ __forceinline__ void delay_entry(const DelayTableParams &p, long long
 // History tail: word w of the new history (32-bit words; every stream's bytes
 // are a multiple of 4 and 4-byte aligned): the last tail_bytes bytes of [old
 // history | chunk] of every stream (the chunk-overlap region of Sec. 3.1, kept
-// resident on the device instead of copying the next chunk's prefix).
+// resident on the device instead of copying the next chunk's prefix). The
+// words of a history fit 32 bits; those of a chunk do not (the down-converter
+// takes up to 2^34 samples, 5.4e9 words of a stream).
 __device__ __forceinline__ void tail_words(const uint8_t *hist_in, const uint8_t *chunk, uint8_t *hist_out,
                                            long long tail_bytes, long long chunk_bytes, int n_streams, int block,
                                            int n_blocks) {
-    const unsigned tw = (unsigned)(tail_bytes >> 2), cw = (unsigned)(chunk_bytes >> 2);
+    const unsigned tw = (unsigned)(tail_bytes >> 2);
+    const long long cw = chunk_bytes >> 2;
     const uint32_t *hi = reinterpret_cast<const uint32_t *>(hist_in), *ch = reinterpret_cast<const uint32_t *>(chunk);
     uint32_t *ho = reinterpret_cast<uint32_t *>(hist_out);
     for (int st = 0; st < n_streams; st++) {
-        const uint32_t *h = hi + (long long)st * tw, *c = ch + (long long)st * cw;
+        // word w comes from word w + cw of [history | chunk]: history words below keep, chunk words from it on
+        const unsigned keep = cw < (long long)tw ? tw - (unsigned)cw : 0u;
+        const uint32_t *h = hi + (long long)st * tw + (keep ? cw : 0), *c = ch + (long long)st * cw + (cw - (long long)tw);
         uint32_t *o = ho + (long long)st * tw;
-        for (unsigned w = (unsigned)block * blockDim.x + threadIdx.x; w < tw; w += (unsigned)n_blocks * blockDim.x) {
-            const unsigned src = w + cw;
-            o[w] = src < tw ? h[src] : c[src - tw];
-        }
+        for (unsigned w = (unsigned)block * blockDim.x + threadIdx.x; w < tw; w += (unsigned)n_blocks * blockDim.x)
+            o[w] = w < keep ? h[w] : c[w];
     }
 }
 
