@@ -47,6 +47,7 @@
 
 #include "fe_device.cuh"
 #include "fe_internal.cuh"
+#include "fe_waits.cuh"
 
 namespace fe {
 
@@ -1015,15 +1016,18 @@ __global__ void __launch_bounds__(kTsThreads, 1) k_phase1_ts(const __grid_consta
             if (nact == 0 || !ok) break;
             if (warp >= 4 && warp < 8) {
                 // ---------------- fill ----------------
-                // a warp that has given up tells the others here, before any of them waits for it
-                int go = ok;
-                asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.s32 q, %1, 0;\n\tbar.red.and.pred q, 1, %2, q;\n\t"
-                             "selp.s32 %0, 1, 0, q;\n\t}\n"
-                             : "=r"(go)
-                             : "r"(go), "n"(kTsFill)
-                             : "memory");
-                ok = go != 0;
-                if (!moved) {
+                // the four warps leave together (ts_fill_round)
+                auto vote = [&](bool mine) -> bool {
+                    int go;
+                    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.s32 q, %1, 0;\n\tbar.red.and.pred q, 1, %2, q;\n\t"
+                                 "selp.s32 %0, 1, 0, q;\n\t}\n"
+                                 : "=r"(go)
+                                 : "r"((int)mine), "n"(kTsFill)
+                                 : "memory");
+                    return go != 0;
+                };
+                auto copy = [&]() -> bool {
+                    bool go = true;
                     // a sequence starts at row 8 (m0 + q0) - rb, 16-byte aligned, of column t + c0 - c (the
                     // columns are laid out at delay c0); one bulk copy per plane, each warp its own tile
 #pragma unroll
@@ -1033,10 +1037,10 @@ __global__ void __launch_bounds__(kTsThreads, 1) k_phase1_ts(const __grid_consta
                         const bool act = ps.ra < ps.rows;
                         const uint16_t *col =
                             p.cols + ((long long)ps.st * P + t2 + (ps.c0 - ps.c)) * p.RTP + (8LL * (p.m0 + ps.q0) - p.rb);
-                        for (int k = 0; k < NST && ok; k++) {
+                        for (int k = 0; k < NST && go; k++) {
                             const unsigned n = ns + (unsigned)k, s = n % NS;
-                            ok = n < NS || wait_bar(&empty[s], ((n / NS) - 1) & 1);
-                            if (!ok) break;
+                            go = n < NS || wait_bar(&empty[s], ((n / NS) - 1) & 1);
+                            if (!go) break;
                             if (!act) {
                                 arrive(&full[s]);
                                 continue;
@@ -1054,77 +1058,72 @@ __global__ void __launch_bounds__(kTsThreads, 1) k_phase1_ts(const __grid_consta
                         }
                     }
                     __syncwarp();
-                    ok = __shfl_sync(0xFFFFFFFFu, (int)ok, 0) != 0;
-                } else {
-                    for (int k = 0; k < NST && ok; k++) {
-                        const unsigned n = ns + (unsigned)k, s = n % NS;
-                        // the decision to go on is the same in every fill thread
-                        go = ft != 0 || n < NS || wait_bar(&empty[s], ((n / NS) - 1) & 1);
-                        asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.s32 q, %1, 0;\n\tbar.red.and.pred q, 1, %2, q;\n\t"
-                                     "selp.s32 %0, 1, 0, q;\n\t}\n"
-                                     : "=r"(go)
-                                     : "r"(go), "n"(kTsFill)
-                                     : "memory");
-                        ok = go != 0;
-                        if (!ok) break;
+                    return __shfl_sync(0xFFFFFFFFu, (int)go, 0) != 0;
+                };
+                auto stage_free = [&](int k) -> bool {
+                    const unsigned n = ns + (unsigned)k;
+                    return ft != 0 || n < NS || wait_bar(&empty[n % NS], ((n / NS) - 1) & 1);
+                };
+                auto realign = [&](int k) {
+                    const unsigned s = (ns + (unsigned)k) % NS;
 #pragma unroll 1
-                        for (int i = 0; i < SJ; i++) {
-                            const int c = (k * SJ + i) / R, j = (k * SJ + i) % R;
-                            const long long t = t2 + c + (long long)N2 * j;   // physical column
+                    for (int i = 0; i < SJ; i++) {
+                        const int c = (k * SJ + i) / R, j = (k * SJ + i) % R;
+                        const long long t = t2 + c + (long long)N2 * j;   // physical column
 #pragma unroll
-                            for (int g = 0; g < G; g++) {
-                                const TsTile &ps = tl[g];
-                                if (ps.ra >= ps.rows) continue;
-                                uint8_t *xb = smem + s * ST + SJ * BB + (i * G + g) * AB;
-                                // 16-byte chunks from the aligned element row0 - sh, each output chunk 16 bytes
-                                // at byte offset 2 sh of two consecutive source chunks
-                                const long long a0 = (long long)p.N * (p.m0 + ps.q0) - ps.c + ps.c0 + t;
-                                const long long ra = floor_div(a0, P);
-                                const long long row0 = ra - p.rb;
-                                const uint16_t *src =
-                                    p.cols + ((long long)ps.st * P + (a0 - ra * P)) * p.RTP + (row0 & ~7LL);
-                                const int sh = (int)(row0 & 7);
-                                constexpr int CPC = XL / 8;
-                                for (int e = ft; e < NPL * CPC; e += kTsFill) {
-                                    const int pl = e / CPC, q8 = e - pl * CPC;
-                                    const uint4 *q = reinterpret_cast<const uint4 *>(src + pl * p.plane_elems) + q8;
-                                    const uint4 v0 = ld_dep(q), v1 = ld_dep(q + 1);
-                                    const uint32_t w[8] = {v0.x, v0.y, v0.z, v0.w, v1.x, v1.y, v1.z, v1.w};
-                                    const uint32_t sel = (sh & 1) ? 0x5432u : 0x3210u;   // 2-byte shift for odd sh
-                                    uint32_t o[4];
+                        for (int g = 0; g < G; g++) {
+                            const TsTile &ps = tl[g];
+                            if (ps.ra >= ps.rows) continue;
+                            uint8_t *xb = smem + s * ST + SJ * BB + (i * G + g) * AB;
+                            // 16-byte chunks from the aligned element row0 - sh, each output chunk 16 bytes
+                            // at byte offset 2 sh of two consecutive source chunks
+                            const long long a0 = (long long)p.N * (p.m0 + ps.q0) - ps.c + ps.c0 + t;
+                            const long long ra = floor_div(a0, P);
+                            const long long row0 = ra - p.rb;
+                            const uint16_t *src =
+                                p.cols + ((long long)ps.st * P + (a0 - ra * P)) * p.RTP + (row0 & ~7LL);
+                            const int sh = (int)(row0 & 7);
+                            constexpr int CPC = XL / 8;
+                            for (int e = ft; e < NPL * CPC; e += kTsFill) {
+                                const int pl = e / CPC, q8 = e - pl * CPC;
+                                const uint4 *q = reinterpret_cast<const uint4 *>(src + pl * p.plane_elems) + q8;
+                                const uint4 v0 = ld_dep(q), v1 = ld_dep(q + 1);
+                                const uint32_t w[8] = {v0.x, v0.y, v0.z, v0.w, v1.x, v1.y, v1.z, v1.w};
+                                const uint32_t sel = (sh & 1) ? 0x5432u : 0x3210u;   // 2-byte shift for odd sh
+                                uint32_t o[4];
 #pragma unroll
-                                    for (int m = 0; m < 4; m++) {
-                                        uint32_t lo = w[m], hi = w[m + 1];
-                                        if ((sh >> 1) == 1) lo = w[m + 1], hi = w[m + 2];
-                                        else if ((sh >> 1) == 2) lo = w[m + 2], hi = w[m + 3];
-                                        else if ((sh >> 1) == 3) lo = w[m + 3], hi = w[m + 4];
-                                        o[m] = __byte_perm(lo, hi, sel);
-                                    }
-                                    reinterpret_cast<uint4 *>(xb + pl * XL * 2)[q8] = make_uint4(o[0], o[1], o[2], o[3]);
+                                for (int m = 0; m < 4; m++) {
+                                    uint32_t lo = w[m], hi = w[m + 1];
+                                    if ((sh >> 1) == 1) lo = w[m + 1], hi = w[m + 2];
+                                    else if ((sh >> 1) == 2) lo = w[m + 2], hi = w[m + 3];
+                                    else if ((sh >> 1) == 3) lo = w[m + 3], hi = w[m + 4];
+                                    o[m] = __byte_perm(lo, hi, sel);
                                 }
-                                if (p.window_tap) {
-                                    // debug tap: the first FIR tap of spectrum q0 + v / 8 at offset P (v % 8) + t
-                                    asm volatile("bar.sync 1, %0;" ::"n"(kTsFill) : "memory");
-                                    const uint16_t *xv = reinterpret_cast<const uint16_t *>(xb);
-                                    for (int vv = ft; vv < 8 * kTcRows; vv += kTsFill) {
-                                        const int mrow = vv >> 3;
-                                        if (mrow < ps.ra || mrow >= ps.rb) continue;
-                                        float x;
-                                        if constexpr (PREC == 2)
-                                            x = __bfloat162float(__ushort_as_bfloat16(xv[vv])) +
-                                                __bfloat162float(__ushort_as_bfloat16(xv[XL + vv]));
-                                        else x = __half2float(__ushort_as_half(xv[vv]));
-                                        p.window_tap[((long long)ps.st * p.M + ps.q0 + mrow) * p.N +
-                                                     (long long)P * (vv & 7) + t] = (int)x;
-                                    }
+                                reinterpret_cast<uint4 *>(xb + pl * XL * 2)[q8] = make_uint4(o[0], o[1], o[2], o[3]);
+                            }
+                            if (p.window_tap) {
+                                // debug tap: the first FIR tap of spectrum q0 + v / 8 at offset P (v % 8) + t
+                                asm volatile("bar.sync 1, %0;" ::"n"(kTsFill) : "memory");
+                                const uint16_t *xv = reinterpret_cast<const uint16_t *>(xb);
+                                for (int vv = ft; vv < 8 * kTcRows; vv += kTsFill) {
+                                    const int mrow = vv >> 3;
+                                    if (mrow < ps.ra || mrow >= ps.rb) continue;
+                                    float x;
+                                    if constexpr (PREC == 2)
+                                        x = __bfloat162float(__ushort_as_bfloat16(xv[vv])) +
+                                            __bfloat162float(__ushort_as_bfloat16(xv[XL + vv]));
+                                    else x = __half2float(__ushort_as_half(xv[vv]));
+                                    p.window_tap[((long long)ps.st * p.M + ps.q0 + mrow) * p.N +
+                                                 (long long)P * (vv & 7) + t] = (int)x;
                                 }
                             }
                         }
-                        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                        asm volatile("bar.sync 1, %0;" ::"n"(kTsFill) : "memory");
-                        if (lane == 0 && warp < 4 + G) arrive(&full[s]);
                     }
-                }
+                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                    asm volatile("bar.sync 1, %0;" ::"n"(kTsFill) : "memory");
+                    if (lane == 0 && warp < 4 + G) arrive(&full[s]);
+                };
+                ok = ts_fill_round<NST>(moved, copy, stage_free, realign, vote);
             } else if (warp == 9) {
                 // ---------------- operand blocks ----------------
                 if (lane == 0) {
