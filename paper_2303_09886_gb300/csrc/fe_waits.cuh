@@ -27,4 +27,40 @@ __host__ __device__ __forceinline__ bool ts_fill_round(bool moved, Copy &&copy, 
     return true;
 }
 
+// A warp's copies into its one buffer, one on its way at a time, and the waits
+// for them. After a wait that gave up (over() ended it) the warp takes no more
+// copies and waits no more: its barrier's phase is not over, so another copy
+// asked for on it would be counted wrongly, and a wait per item left would
+// each run to its limit.
+struct CopyWait {
+    unsigned parity = 0;
+    bool pending = false, dead = false;
+    template <class Start>
+    __host__ __device__ __forceinline__ void ask(Start &&start) {
+        if (dead) return;
+        start();
+        pending = true;
+    }
+    // here(parity): whether the copy has arrived; over(): whether to give up. False: the buffer holds nothing.
+    template <class Here, class Over>
+    __host__ __device__ __forceinline__ bool arrived(Here &&here, Over &&over) {
+        if (dead) return false;
+        while (!here(parity))
+            if (over()) {
+                dead = true;
+                return false;
+            }
+        parity ^= 1u;
+        pending = false;
+        return true;
+    }
+    // before the warp leaves: a copy still on its way (there is none unless a wait gave up) is given one more limit
+    template <class Here, class Over>
+    __host__ __device__ __forceinline__ void leave(Here &&here, Over &&over) {
+        if (pending)
+            while (!here(parity))
+                if (over()) return;
+    }
+};
+
 }  // namespace fe

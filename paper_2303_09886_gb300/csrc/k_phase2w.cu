@@ -43,6 +43,7 @@
 
 #include "fe_device.cuh"
 #include "fe_internal.cuh"
+#include "fe_waits.cuh"
 
 namespace fe {
 
@@ -96,6 +97,7 @@ struct WSmem {
     float4 q[kWWarps][32];                // per warp: Q[d]
     unsigned long long full[kWWarps];     // per warp: its pair has arrived
     int seg_end;
+    int gave_up;                          // a warp's wait has: the others do not wait to their limits
 };
 
 }  // namespace
@@ -146,6 +148,7 @@ __global__ void __launch_bounds__(kWThreads, 1) k_phase2w(const __grid_constant_
     const int grp = warp >> 2, pr = (warp >> 1) & 1, pol = warp & 1;
     float4(*tile)[33] = sm.buf[warp];
     const uint32_t mbar = sm_addr(&sm.full[warp]);
+    if (threadIdx.x == 0) sm.gave_up = 0;   // (read after the first segment's barriers)
     if (lane == 0) {
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(mbar));
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -206,11 +209,35 @@ __global__ void __launch_bounds__(kWThreads, 1) k_phase2w(const __grid_constant_
     pdl_release();
     pdl_wait();   // phase 1's results, and the delay table's
     asm volatile("" : "+l"(ftab), "+l"(gtab)::"memory");
+    // the warp's waits, the same in all its lanes (bounded: fengine_device_status reports one that gave up)
+    CopyWait cw;
+    long long t0 = 0;
+    auto here = [&](unsigned parity) -> bool {
+        uint32_t ok;
+        asm volatile(
+            "{\n\t.reg .pred q;\n\tmbarrier.try_wait.parity.shared::cta.b64 q, [%1], %2, %3;\n\t"
+            "selp.u32 %0, 1, 0, q;\n\t}\n"
+            : "=r"(ok)
+            : "r"(mbar), "r"(parity), "r"(20000u)
+            : "memory");
+        return __all_sync(0xFFFFFFFFu, ok != 0) != 0;
+    };
+    auto late = [&]() -> bool { return __any_sync(0xFFFFFFFFu, clock64() - t0 > kWaitCycles) != 0; };
+    auto over = [&]() -> bool {
+        if (__any_sync(0xFFFFFFFFu, *(volatile int *)&sm.gave_up != 0)) return true;
+        if (!late()) return false;
+        if (lane == 0) {
+            *(volatile int *)&sm.gave_up = 1;
+            if (p.err) atomicExch(p.err, 2);
+        }
+        return true;
+    };
     if (it0 + grp < it1 && active_in(nx)) {
-        if (lane == 0) fetch(nx);
+        cw.ask([&] {
+            if (lane == 0) fetch(nx);
+        });
         model(nx);
     }
-    uint32_t parity = 0;
 
     for (int seg = it0; seg < it1;) {
         // [seg, se): items of one class and antenna whose first spectra use the same gain sets
@@ -252,7 +279,7 @@ __global__ void __launch_bounds__(kWThreads, 1) k_phase2w(const __grid_constant_
         for (int it = first; it < se; it += kWGroups) {
             const int q0 = q_first + (it - first) * kWR;
             const int Rv = min(kWR, p.q_begin + p.q_count - q0);
-            const bool active = 2 * pr < Rv;
+            bool active = 2 * pr < Rv;
             advance(nx);   // the group's next item
             const bool more = it + kWGroups < it1 && active_in(nx);
 
@@ -278,24 +305,11 @@ __global__ void __launch_bounds__(kWThreads, 1) k_phase2w(const __grid_constant_
                 Pu = cmulp_conj(cpair{make_float2(c0, c1), make_float2(s0, s1)}, P);
             }
             cpair z[32];
+            if (active) {   // the pair has arrived
+                t0 = clock64();
+                active = cw.arrived(here, over);
+            }
             if (active) {
-                // the pair has arrived (a bounded wait: fengine_device_status reports one that gave up)
-                const long long t0 = clock64();
-                for (;;) {
-                    uint32_t ok;
-                    asm volatile(
-                        "{\n\t.reg .pred q;\n\tmbarrier.try_wait.parity.shared::cta.b64 q, [%1], %2, %3;\n\t"
-                        "selp.u32 %0, 1, 0, q;\n\t}\n"
-                        : "=r"(ok)
-                        : "r"(mbar), "r"(parity), "r"(20000u)
-                        : "memory");
-                    if (ok) break;
-                    if (clock64() - t0 > kWaitCycles) {
-                        if (p.err) atomicExch(p.err, 2);
-                        break;
-                    }
-                }
-                parity ^= 1u;
                 const float4 *lin = &tile[0][0];
                 if constexpr (IN == kInPairs) {
 #pragma unroll
@@ -338,7 +352,9 @@ __global__ void __launch_bounds__(kWThreads, 1) k_phase2w(const __grid_constant_
             __syncwarp();
             const int gcur = gsel;
             if (more) {
-                if (lane == 0) fetch(nx);
+                cw.ask([&] {
+                    if (lane == 0) fetch(nx);
+                });
                 model(nx);
             }
             if (active) fft_regc2<32>(z);                         // z[d] = F[lane + 32 d]
@@ -448,6 +464,8 @@ __global__ void __launch_bounds__(kWThreads, 1) k_phase2w(const __grid_constant_
         }
         seg = se;
     }
+    t0 = clock64();
+    cw.leave(here, late);
 }
 
 long long phase2w_items(const Phase2Params &p, int n_ant) {
