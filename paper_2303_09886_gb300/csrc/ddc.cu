@@ -46,7 +46,8 @@ struct DdcParams {
     long long L, H;                // chunk and history samples (H a multiple of 16, >= Lh)
     long long t_in;                // first input sample of the chunk
     long long j0;                  // first output of the call (= 2 t_in / D)
-    int Th2, Lout;                 // Lh / (D / 2), outputs per stream
+    int Th2;                       // Lh / (D / 2)
+    long long Lout;                // outputs per stream (up to 2^34)
     const float2 *taps;            // [Lh] h[u] exp(2 pi i fc u)
     double fc;
     float g2;                      // 2 g
@@ -222,7 +223,7 @@ __global__ void __launch_bounds__(ddc_threads(D2)) k_ddc(const __grid_constant__
         q[r] = (unsigned)(int)rr & 0x3FFu;
         if (p.out_float && k0 + r < p.Lout) p.out_float[(long long)st * p.Lout + k0 + r] = y;
     }
-    uint8_t *o = p.out + (long long)st * (5LL * p.Lout / 4) + 5 * (k0 >> 2);
+    uint8_t *o = p.out + (long long)st * (5 * p.Lout / 4) + 5 * (k0 >> 2);
     if (k0 + kDdcPer <= p.Lout && ((uintptr_t)o & 3u) == 0) {
         // 16 fields of 10 bits as five big-endian words
         const uint32_t w[5] = {q[0] << 22 | q[1] << 12 | q[2] << 2 | q[3] >> 8,
@@ -398,7 +399,7 @@ extern "C" fengine_status fengine_ddc_process(fengine_ddc_t d, void *cuda_stream
     p.t_in = first_sample;
     p.j0 = first_sample / (d->D / 2);
     p.Th2 = d->Lh / (d->D / 2);
-    p.Lout = (int)(d->L / (d->D / 2));
+    p.Lout = d->L / (d->D / 2);
     p.taps = d->d_taps;
     p.fc = d->fc;
     p.g2 = 2.0f * d->g;
