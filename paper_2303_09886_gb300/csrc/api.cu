@@ -325,44 +325,6 @@ fengine_status fengine_plan_create(const fengine_config *cfg, fengine_plan_t *ou
         release(pl);
         return cuda_fail(e, "kernel attributes");
     }
-    // Slab of spectra per phase-1 / phase-2 launch pair: built-in, the
-    // spectra whose intermediate (all streams) is about 3 GiB, a multiple of
-    // 32 (both phases' tiles): the whole chunk of every workload here, in one
-    // buffer and one launch pair. Neither phase is bound by memory (the second
-    // stage takes the same time per spectrum from L2), so smaller slabs only
-    // add launches and tails: 8192 channels, 4 antennas x 2 x 2^25 samples
-    // take 0.89 ms as one slab and 1.02 ms as five of 256 MiB. Of the
-    // device's free memory a slab takes 1/32 at most, so that many plans fit
-    // side by side; the least is the 256 MiB slab.
-    // intermediate element: FP32 (re, im), or FP16 (re, im) in the FP16 form
-    pl->a_elem = pl->precision == FENGINE_TC_FP16 ? 4 : 8;
-    const size_t per_spec = (size_t)ns * (pl->N1 / 2 + 1) * pl->N2 * pl->a_elem;
-    const long long M32 = (M + 31) / 32 * 32;
-    auto slab_of = [&](size_t bytes) {
-        long long s = (long long)(bytes / per_spec) / 32 * 32;
-        if (s < 32) s = 32;
-        return s > M32 ? M32 : s;
-    };
-    const long long SL_min = slab_of((size_t)256 << 20);
-    size_t mem_free = 0, mem_total = 0;
-    if (cudaMemGetInfo(&mem_free, &mem_total) != cudaSuccess) mem_free = 0;
-    const long long SL_max = std::max(SL_min, slab_of(std::min((size_t)3 << 30, mem_free / 32)));
-    long long SL = cfg->slab_spectra ? (cfg->slab_spectra > M32 ? M32 : cfg->slab_spectra) : SL_max;
-    size_t a_bytes = 0;
-    for (;;) {
-        a_bytes = (size_t)((M + SL - 1) / SL > 1 ? 2 : 1) * SL * per_spec;
-        e = dalloc(pl, &pl->d_A, a_bytes);
-        if (e == cudaSuccess || cfg->slab_spectra || SL <= SL_min) break;
-        cudaGetLastError();
-        SL = SL / 64 * 32 > SL_min ? SL / 64 * 32 : SL_min;
-    }
-    if (e != cudaSuccess) {
-        release(pl);
-        g_last_error = std::string("device allocation: ") + cudaGetErrorString(e);
-        return FENGINE_ENOMEM;
-    }
-    pl->SL = (int)SL;
-    pl->n_slabs = (int)((M + SL - 1) / SL);
     if ((e = dalloc(pl, &pl->d_w, sizeof(float) * N * T)) != cudaSuccess ||
         (e = dalloc(pl, &pl->d_tw1, sizeof(float2) * (pl->N1 / 2 + 1) * pl->N2)) != cudaSuccess ||
         (e = dalloc(pl, &pl->d_tw2, sizeof(float2) * pl->N2)) != cudaSuccess ||
@@ -384,7 +346,7 @@ fengine_status fengine_plan_create(const fengine_config *cfg, fengine_plan_t *ou
         g_last_error = std::string("device allocation: ") + cudaGetErrorString(e);
         return FENGINE_ENOMEM;
     }
-    pl->scratch_bytes = a_bytes + sizeof(float2) * ns * M + sizeof(int) * ns * M;
+    pl->scratch_bytes = sizeof(float2) * ns * M + sizeof(int) * ns * M;
     if ((e = cudaMallocHost((void **)&pl->h_seg, sizeof(DelaySeg) * fe::kMaxSeg * ns)) != cudaSuccess ||
         (e = cudaMallocHost((void **)&pl->h_nseg, sizeof(int) * ns)) != cudaSuccess ||
         (e = cudaMallocHost((void **)&pl->h_gains, sizeof(float2) * ns * fe::kMaxGainSeg * n)) != cudaSuccess ||
@@ -459,6 +421,46 @@ fengine_status fengine_plan_create(const fengine_config *cfg, fengine_plan_t *ou
         // (column group, k1-slice, item) passes
         pl->tc_splits = sms > 0 ? sms : 148;
     }
+    // Slab of spectra per phase-1 / phase-2 launch pair: built-in, the
+    // spectra whose intermediate (all streams) is about 3 GiB, a multiple of
+    // 32 (both phases' tiles): the whole chunk of every workload here, in one
+    // buffer and one launch pair. Neither phase is bound by memory (the second
+    // stage takes the same time per spectrum from L2), so smaller slabs only
+    // add launches and tails: 8192 channels, 4 antennas x 2 x 2^25 samples
+    // take 0.89 ms as one slab and 1.02 ms as five of 256 MiB. Of the
+    // device's free memory a slab takes 1/32 at most, so that many plans fit
+    // side by side; the least is the 256 MiB slab. The plan's last allocation:
+    // it takes less where the device has no room for it next to the rest.
+    // intermediate element: FP32 (re, im), or FP16 (re, im) in the FP16 form
+    pl->a_elem = pl->precision == FENGINE_TC_FP16 ? 4 : 8;
+    const size_t per_spec = (size_t)ns * (pl->N1 / 2 + 1) * pl->N2 * pl->a_elem;
+    const long long M32 = (M + 31) / 32 * 32;
+    auto slab_of = [&](size_t bytes) {
+        long long s = (long long)(bytes / per_spec) / 32 * 32;
+        if (s < 32) s = 32;
+        return s > M32 ? M32 : s;
+    };
+    const long long SL_min = slab_of((size_t)256 << 20);
+    size_t mem_free = 0, mem_total = 0;
+    if (cudaMemGetInfo(&mem_free, &mem_total) != cudaSuccess) mem_free = 0;
+    const long long SL_max = std::max(SL_min, slab_of(std::min((size_t)3 << 30, mem_free / 32)));
+    long long SL = cfg->slab_spectra ? (cfg->slab_spectra > M32 ? M32 : cfg->slab_spectra) : SL_max;
+    size_t a_bytes = 0;
+    for (;;) {
+        a_bytes = (size_t)((M + SL - 1) / SL > 1 ? 2 : 1) * SL * per_spec;
+        e = dalloc(pl, &pl->d_A, a_bytes);
+        if (e == cudaSuccess || cfg->slab_spectra || SL <= SL_min) break;
+        cudaGetLastError();
+        SL = SL / 64 * 32 > SL_min ? SL / 64 * 32 : SL_min;
+    }
+    if (e != cudaSuccess) {
+        release(pl);
+        g_last_error = std::string("device allocation: ") + cudaGetErrorString(e);
+        return FENGINE_ENOMEM;
+    }
+    pl->scratch_bytes += a_bytes;
+    pl->SL = (int)SL;
+    pl->n_slabs = (int)((M + SL - 1) / SL);
     // twiddles, evaluated in FP64 with exact integer phase reduction
     std::vector<float2> tw1((size_t)(pl->N1 / 2 + 1) * pl->N2), tw2(pl->N2);
     for (int k1 = 0; k1 <= pl->N1 / 2; k1++)
