@@ -440,18 +440,24 @@ fengine_status fengine_plan_create(const fengine_config *cfg, fengine_plan_t *ou
         if (s < 32) s = 32;
         return s > M32 ? M32 : s;
     };
+    // as many slabs as that takes, of equal size (a call just over one slab would
+    // otherwise hold a second, nearly unused buffer)
+    auto even = [&](long long s) {
+        const long long k = (M + s - 1) / s;
+        return ((M + k - 1) / k + 31) / 32 * 32;
+    };
     const long long SL_min = slab_of((size_t)256 << 20);
     size_t mem_free = 0, mem_total = 0;
     if (cudaMemGetInfo(&mem_free, &mem_total) != cudaSuccess) mem_free = 0;
     const long long SL_max = std::max(SL_min, slab_of(std::min((size_t)3 << 30, mem_free / 32)));
-    long long SL = cfg->slab_spectra ? (cfg->slab_spectra > M32 ? M32 : cfg->slab_spectra) : SL_max;
+    long long SL = cfg->slab_spectra ? (cfg->slab_spectra > M32 ? M32 : cfg->slab_spectra) : even(SL_max);
     size_t a_bytes = 0;
     for (;;) {
         a_bytes = (size_t)((M + SL - 1) / SL > 1 ? 2 : 1) * SL * per_spec;
         e = dalloc(pl, &pl->d_A, a_bytes);
         if (e == cudaSuccess || cfg->slab_spectra || SL <= SL_min) break;
         cudaGetLastError();
-        SL = SL / 64 * 32 > SL_min ? SL / 64 * 32 : SL_min;
+        SL = SL / 64 * 32 > SL_min ? even(SL / 64 * 32) : SL_min;
     }
     if (e != cudaSuccess) {
         release(pl);

@@ -1,6 +1,6 @@
 """The memory a plan takes: one that fits with slabs of 256 MiB is made, however
 little the device has left beside it (the built-in slab gives way, the rest of
-the plan does not)."""
+the plan does not), and the slabs of a call that takes several are even."""
 import pytest
 
 from paper_2303_09886_gb300 import fengine
@@ -31,3 +31,17 @@ def test_plan_next_to_little_free_memory():
     finally:
         del fill
         torch.cuda.empty_cache()
+
+
+@pytest.mark.parametrize("precision", [fengine.FP32, fengine.TC_FP16])
+def test_slabs_are_even(precision):
+    n, ants = 8192, 8
+    per_spectrum = 2 * ants * 9 * 1024 * (8 if precision == fengine.FP32 else 4)
+    M = (3 << 30) // per_spectrum + 40                     # a little more than 3 GiB of intermediate
+    plan = fengine.Plan(ants, n, 4, 2 * n * M, precision=precision)
+    k, slab = int(plan.info.slabs_per_chunk), int(plan.info.slab_spectra)
+    bytes_ = int(plan.info.scratch_bytes)
+    plan.close()
+    assert k >= 2 and slab % 32 == 0 and k * slab < M + 32 * k
+    if precision == fengine.FP32:
+        assert bytes_ < 2 * slab * per_spectrum + (1 << 20)
