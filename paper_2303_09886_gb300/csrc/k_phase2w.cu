@@ -103,10 +103,15 @@ struct WSmem {
 }  // namespace
 
 // Persistent: one CTA per SM (a thread holds 32 points of two spectra: 128
-// registers of data), a contiguous range of work items of equal work per CTA. The CTAs of one (CAP = 1) or several plans' second
-// stages in one grid: member m owns CTAs [start[m], start[m + 1]) and aux[m]
-// antennas.
-template <int IN, int CAP>
+// registers of data), a contiguous range of work items of equal work per CTA.
+// The CTAs of one (CAP = 1) or several plans' second stages in one grid:
+// member m owns CTAs [start[m], start[m + 1]) and aux[m] antennas. kPre: the
+// spectra before quantisation are written as well, by a kernel of its own
+// (512 spectra, 2 polarisations of 8192 channels: 125 us, and 173 where the
+// one kernel did it in a loop over slots with the points in local memory; with
+// the stores in a second copy of the epilogue the plain one took 490 us
+// instead of 453 on the workload above).
+template <int IN, int CAP, bool kPre>
 __global__ void __launch_bounds__(kWThreads, 1) k_phase2w(const __grid_constant__ GroupArgs<Phase2Params, CAP> ga) {
     constexpr bool kPaired = IN == kInPairs || IN == kInHalfPairs, kHalf = IN == kInHalf || IN == kInHalfPairs;
     extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -211,7 +216,7 @@ __global__ void __launch_bounds__(kWThreads, 1) k_phase2w(const __grid_constant_
     asm volatile("" : "+l"(ftab), "+l"(gtab)::"memory");
     // the warp's waits, the same in all its lanes (bounded: fengine_device_status reports one that gave up)
     CopyWait cw;
-    long long t0 = 0;
+    long long t0 = 0;   // of the first failed try
     auto here = [&](unsigned parity) -> bool {
         uint32_t ok;
         asm volatile(
@@ -222,7 +227,10 @@ __global__ void __launch_bounds__(kWThreads, 1) k_phase2w(const __grid_constant_
             : "memory");
         return __all_sync(0xFFFFFFFFu, ok != 0) != 0;
     };
-    auto late = [&]() -> bool { return __any_sync(0xFFFFFFFFu, clock64() - t0 > kWaitCycles) != 0; };
+    auto late = [&]() -> bool {
+        if (t0 == 0) t0 = clock64();
+        return __any_sync(0xFFFFFFFFu, clock64() - t0 > kWaitCycles) != 0;
+    };
     auto over = [&]() -> bool {
         if (__any_sync(0xFFFFFFFFu, *(volatile int *)&sm.gave_up != 0)) return true;
         if (!late()) return false;
@@ -306,7 +314,7 @@ __global__ void __launch_bounds__(kWThreads, 1) k_phase2w(const __grid_constant_
             }
             cpair z[32];
             if (active) {   // the pair has arrived
-                t0 = clock64();
+                t0 = 0;
                 active = cw.arrived(here, over);
             }
             if (active) {
@@ -363,28 +371,35 @@ __global__ void __launch_bounds__(kWThreads, 1) k_phase2w(const __grid_constant_
                 const float4 *qs = sm.q[warp], *gp = sm.gain[pol] + lane;
                 unsigned *stg = sm.stg[grp][pol];
                 const int q = q0 + 2 * pr, gst = pol ? gs1 : gs0;
-                if (gcur == (gst | gst << 8) && !p.prequant) {
+                float2 *pre = kPre ? p.prequant + ((long long)stream * M + q) * n : nullptr;
+                const bool two = 2 * pr + 1 < Rv;
+                auto put = [&](int k2, int k, const cpair &y) {
+                    if constexpr (kPre) {
+                        pre[k] = make_float2(y.x.x, y.y.x);
+                        if (two) pre[n + k] = make_float2(y.x.y, y.y.y);
+                    }
+                    stg[stg_word(k2, pr)] = quant8x4(make_float2(y.x.x, y.y.x), make_float2(y.x.y, y.y.y));
+                };
+                if (gcur == (gst | gst << 8)) {
 #pragma unroll
                     for (int d = 0; d < 16; d++) {   // channel k1 + N1 k2
+                        const int k2 = lane + 32 * d;
                         const cpair r = cmulp<true>(P, as_cpair(qs[d]));
-                        const cpair y = cmulp<false>(as_cpair(gp[32 * d]), cmulp<false>(r, z[d]));
-                        stg[stg_word(lane + 32 * d, pr)] = quant8x4(make_float2(y.x.x, y.y.x), make_float2(y.x.y, y.y.y));
+                        put(k2, k1 + N1 * k2, cmulp<false>(as_cpair(gp[32 * d]), cmulp<false>(r, z[d])));
                     }
                     if (upper) {
 #pragma unroll
                         for (int d = 16; d < 32; d++) {   // channel N - (k1 + N1 k2)
+                            const int k2 = lane + 32 * d;
                             const cpair r = cmulp_conj(Pu, as_cpair(qs[d]));
-                            const cpair y = cmulp<false>(as_cpair(gp[32 * d]), cmulp_conj(r, z[d]));
-                            stg[stg_word(lane + 32 * d, pr)] =
-                                quant8x4(make_float2(y.x.x, y.y.x), make_float2(y.x.y, y.y.y));
+                            put(k2, N - (k1 + N1 * k2), cmulp<false>(as_cpair(gp[32 * d]), cmulp_conj(r, z[d])));
                         }
                     }
                 } else {
-                    // the same with the spectra before quantisation written out, or with the gains of a
-                    // spectrum whose set is not the segment's (a gain update inside the item)
+                    // the same with the gains of a spectrum whose set is not the segment's (a gain update inside
+                    // the item)
                     const float2 *gd0 = p.gains + ((long long)stream * p.n_gsets_max + (gcur & 0xFF)) * n;
                     const float2 *gd1 = p.gains + ((long long)stream * p.n_gsets_max + (gcur >> 8)) * n;
-                    float2 *pre = p.prequant ? p.prequant + ((long long)stream * M + q) * n : nullptr;
                     cpair zl[32];
 #pragma unroll
                     for (int d = 0; d < 32; d++) zl[d] = z[d];
@@ -396,11 +411,7 @@ __global__ void __launch_bounds__(kWThreads, 1) k_phase2w(const __grid_constant_
                         const cpair v = up ? cmulp_conj(cmulp_conj(Pu, qd), zl[d]) : cmulp<false>(cmulp<true>(P, qd), zl[d]);
                         const float2 a = __ldg(gd0 + k), b = __ldg(gd1 + k);
                         const cpair y = cmulp<false>(cpair{make_float2(a.x, b.x), make_float2(a.y, b.y)}, v);
-                        if (pre) {
-                            pre[k] = make_float2(y.x.x, y.y.x);
-                            if (2 * pr + 1 < Rv) pre[n + k] = make_float2(y.x.y, y.y.y);
-                        }
-                        stg[stg_word(k2, pr)] = quant8x4(make_float2(y.x.x, y.y.x), make_float2(y.x.y, y.y.y));
+                        put(k2, k, y);
                     }
                 }
             }
@@ -464,7 +475,7 @@ __global__ void __launch_bounds__(kWThreads, 1) k_phase2w(const __grid_constant_
         }
         seg = se;
     }
-    t0 = clock64();
+    t0 = 0;
     cw.leave(here, late);
 }
 
@@ -483,12 +494,24 @@ int phase2w_wave() {
 // (g = nullptr: only the kernel's shared-memory size is set)
 template <int IN, int CAP>
 static cudaError_t launch_w(const GroupArgs<Phase2Params, CAP> *g, cudaStream_t s, bool pdl) {
-    if (!g)
-        return cudaFuncSetAttribute(k_phase2w<IN, CAP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(WSmem));
+    void (*kernel)(GroupArgs<Phase2Params, CAP>) = k_phase2w<IN, CAP, false>;
+    if (!g) {
+        const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(WSmem));
+        if constexpr (CAP == 1) {
+            if (e == cudaSuccess)
+                return cudaFuncSetAttribute(k_phase2w<IN, 1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                            (int)sizeof(WSmem));
+        }
+        return e;
+    }
     for (int m = 0; m < g->n; m++)
-        if (g->p[m].N / g->p[m].N1 != kWN2 || g->p[m].a_spectra % 2) return cudaErrorInvalidValue;
+        if (g->p[m].N / g->p[m].N1 != kWN2 || g->p[m].a_spectra % 2 || (CAP > 1 && g->p[m].prequant))
+            return cudaErrorInvalidValue;
     if (g->n < 1 || g->start[g->n] < 1) return cudaSuccess;
-    return launch_kernel(k_phase2w<IN, CAP>, dim3((unsigned)g->start[g->n]), (unsigned)kWThreads, sizeof(WSmem), s, pdl, *g);
+    if constexpr (CAP == 1) {
+        if (g->p[0].prequant) kernel = k_phase2w<IN, 1, true>;
+    }
+    return launch_kernel(kernel, dim3((unsigned)g->start[g->n]), (unsigned)kWThreads, sizeof(WSmem), s, pdl, *g);
 }
 
 template <int CAP>
