@@ -224,6 +224,11 @@ fengine_status process_chunk_deferred(fengine_plan_t pl, cudaStream_t st, const 
 // Tile shapes (host and device agree through these).
 constexpr int kP1Block = 32;   // spectra per block of a phase-1 tile (one DFT stage)
 constexpr int kP1Blocks = 4;   // blocks per phase-1 tile at most
+// Threads of a phase-1 CTA of C columns: one per pair of columns, and no fewer than 64, which the DFT stage of the
+// narrowest tiles (below 256 channels) keeps busy. With 256 for every tile, half a warp in eight filtered there: 16
+// channels, 2^20 spectra in two streams, 2 taps, 841 us a call against 471
+// (16 taps: 1063 and 593).
+constexpr int p1_threads(int C) { return C / 2 > 64 ? C / 2 : 64; }
 int phase1_rows(int T, int N1, int N2, int q_count, int n_streams);   // spectra per phase-1 CTA
 inline int phase1_W(int N1, int N2) {
     int w = 512 / N1;           // 512 FIR columns per tile

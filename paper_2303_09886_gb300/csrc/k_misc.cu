@@ -58,7 +58,8 @@ int phase1_rows(int T, int N1, int N2, int q_count, int n_streams) {
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
         sms = 148;
-    const long long slots = 2LL * sms, cols = (long long)(N2 / phase1_W(N1, N2)) * n_streams;
+    const int W = phase1_W(N1, N2);
+    const long long slots = 512LL / p1_threads(N1 * W) * sms, cols = (long long)(N2 / W) * n_streams;
     int best = kP1Block;
     double best_cost = -1.0;
     for (int rows : {128, 64, 32, 16, 8}) {

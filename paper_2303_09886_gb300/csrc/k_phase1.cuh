@@ -40,7 +40,8 @@
 // intermediate is stored with the streaming hint: plain stores take 0.50 ms,
 // because the lines written push the packed rows out of L2.
 // 32 taps, 8192 channels, 8.4 M samples: 0.074 ms against 0.176 (the second
-// sweep's rows are decoded again, but nothing spills).
+// sweep's rows are decoded again; 32 to 96 bytes spill where one sweep of 32
+// taps spilled 2 to 4 KB).
 #pragma once
 #include <algorithm>
 
@@ -49,13 +50,12 @@
 
 namespace fe {
 
-constexpr int kP1Threads = 256;
-
 template <int T, int N1, int W>
 struct P1Shape {
     static constexpr int C = N1 * W;         // FIR columns per tile
     static constexpr int CW = C < 64 ? C : 64;      // columns of one warp
     static constexpr int NW = C / CW;        // warps that filter
+    static constexpr int THREADS = p1_threads(C), CTAS = 512 / THREADS;   // resident per SM (128 registers each)
     static constexpr int NS = CW / W;        // segments (t1 values) of one warp
     // floats per row pair of g (N1 = 64: a warp of the DFT reads 4 row pairs at a time, half a warp on
     // 32 banks)
@@ -406,18 +406,18 @@ __device__ __forceinline__ void p1_dft(const Phase1Params &p, float *g, const fl
     const long long pair0 = (long long)stream * (p.a_spectra >> 1) + (qa >> 1);
     if constexpr (N1 == 64) {
         // two warps per 32 (row pair, t2): a thread with both halves would need 256 registers
-        static_assert((kP1Block / 2) * W * 2 == kP1Threads, "one pass");
+        static_assert((kP1Block / 2) * W * 2 == S::THREADS, "one pass");
         const int wq = (threadIdx.x >> 5) & 3, e = 32 * wq + (threadIdx.x & 31), rp = e / W, w = e % W;
         const int n = ((rows + 1) >> 1) * W;
         if (32 * wq >= n) return;
         float2 *gp = reinterpret_cast<float2 *>(g + rp * S::GROW) + w;
         float4 *out = reinterpret_cast<float4 *>(p.A) + (pair0 + rp) * (H1 + 1) * N2 + t2_0 + w;
         const float4 *tp = reinterpret_cast<const float4 *>(tw) + w;
-        if (threadIdx.x < kP1Threads / 2) p1_half64<W, 0>(gp, e < n, 1 + wq, tp, out, N2);
+        if (threadIdx.x < S::THREADS / 2) p1_half64<W, 0>(gp, e < n, 1 + wq, tp, out, N2);
         else p1_half64<W, 1>(gp, e < n, 1 + wq, tp, out, N2);
     } else {
 #pragma unroll 1
-        for (int e = threadIdx.x; e < ((rows + 1) >> 1) * W; e += kP1Threads) {
+        for (int e = threadIdx.x; e < ((rows + 1) >> 1) * W; e += S::THREADS) {
             const int rp = e / W, w = e % W;
             const float2 *gp = reinterpret_cast<const float2 *>(g + rp * S::GROW) + w;
             float2 x[N1];
@@ -436,7 +436,7 @@ __device__ __forceinline__ void p1_dft(const Phase1Params &p, float *g, const fl
 // start[m + 1]), decomposed into the (t2 block, spectrum tile, stream) of its
 // own launch.
 template <int T, int N1, int W, int CAP>
-__global__ void __launch_bounds__(kP1Threads, 2) k_phase1(const __grid_constant__ GroupArgs<Phase1Params, CAP> ga) {
+__global__ void __launch_bounds__(P1Shape<T, N1, W>::THREADS, P1Shape<T, N1, W>::CTAS) k_phase1(const __grid_constant__ GroupArgs<Phase1Params, CAP> ga) {
     using S = P1Shape<T, N1, W>;
     extern __shared__ __align__(16) float gs[];   // g, the twiddles, the staged input
     __shared__ int c_sm[kP1Block];
@@ -457,7 +457,7 @@ __global__ void __launch_bounds__(kP1Threads, 2) k_phase1(const __grid_constant_
     const long long rel_base = (long long)N * (p.m0 + q0) - (p.t_in - p.H) + t2_0;
 
     // this tile's twiddles exp(-2 pi i k1 t2 / N) (read after the first block's barrier)
-    for (int i = threadIdx.x; i < (N1 / 2 + 1) * W; i += kP1Threads) {
+    for (int i = threadIdx.x; i < (N1 / 2 + 1) * W; i += S::THREADS) {
         const float2 v = __ldg(p.tw1 + (long long)(i / W) * N2 + t2_0 + i % W);
         reinterpret_cast<float4 *>(tw)[i] = make_float4(v.x, v.x, v.y, v.y);
     }
@@ -616,7 +616,7 @@ cudaError_t launch_phase1_tw(const GroupArgs<Phase1Params, CAP> *g, cudaStream_t
             (g->p[m].rows & 1))
             return cudaErrorInvalidValue;
     if (g->n < 1 || g->start[g->n] < 1) return cudaSuccess;
-    return launch_kernel(k_phase1<T, N1, W, CAP>, dim3((unsigned)g->start[g->n]), (unsigned)kP1Threads, S::SMEM, s, pdl, *g);
+    return launch_kernel(k_phase1<T, N1, W, CAP>, dim3((unsigned)g->start[g->n]), (unsigned)S::THREADS, S::SMEM, s, pdl, *g);
 }
 
 template <int T, int CAP>
