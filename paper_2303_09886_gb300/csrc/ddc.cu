@@ -70,16 +70,15 @@ __host__ __device__ __forceinline__ int ddc_plane_words(int n_out, int Th2) {
     return (ppos(n_out + Th2 + ddc_shift(Th2) + 1) + 1 + 3) & ~3;
 }
 
-// NT taps from a0 + OFF on, a0 a multiple of 16 (h: the plane's taps a0 + OFF
-// ...) for the thread's 16 outputs; w: the plane at element 16 (thread + c)
-// (see ddc_shift). Output r's tap a0 + OFF + aa reads window element NT - 1 -
-// aa + r; taps in ascending order.
-template <int NT, int OFF = 0>
+// NT taps from a0 on (h: the plane's taps a0 ...) for the thread's 16 outputs;
+// w: the plane at element 16 (thread + c) (see ddc_shift). Output r's tap a0 +
+// aa reads window element NT - 1 - aa + r; taps in ascending order.
+template <int NT>
 __device__ __forceinline__ void ddc_block(float2 (&acc)[kDdcPer], const float *w, const float2 *h) {
     float x[kDdcPer + NT - 1];
 #pragma unroll
     for (int i = 0; i < kDdcPer + NT - 1; i++) {
-        const int k = 17 - NT - OFF + i;
+        const int k = 17 - NT + i;
         x[i] = w[k + (k >> 4)];
     }
 #pragma unroll
@@ -185,18 +184,38 @@ __global__ void __launch_bounds__(ddc_threads(D2)) k_ddc(const __grid_constant__
             ddc_block<16>(acc, w, h + a0);
             w -= 17;
         }
-        // what is left of a filter whose length is no multiple of 16 (Th2 is even), in blocks of 8, 4 and 2
-        // (D = 32, 4 and 6 taps per plane, 2^16 samples: 36.0 and 39.1 us a call with a loop over single taps)
-        switch ((Th2 - a0) >> 1) {
-            case 1: ddc_block<2>(acc, w, h + a0); break;
-            case 2: ddc_block<4>(acc, w, h + a0); break;
-            case 3: ddc_block<4>(acc, w, h + a0), ddc_block<2, 4>(acc, w, h + a0 + 4); break;
-            case 4: ddc_block<8>(acc, w, h + a0); break;
-            case 5: ddc_block<8>(acc, w, h + a0), ddc_block<2, 8>(acc, w, h + a0 + 8); break;
-            case 6: ddc_block<8>(acc, w, h + a0), ddc_block<4, 8>(acc, w, h + a0 + 8); break;
-            case 7:
-                ddc_block<8>(acc, w, h + a0), ddc_block<4, 8>(acc, w, h + a0 + 8), ddc_block<2, 12>(acc, w, h + a0 + 12);
-                break;
+        if (a0 + 8 <= Th2) {
+            ddc_block<8>(acc, w, h + a0);
+            a0 += 8;
+        }
+        if constexpr (D2 == 16) {
+            // what is left of a filter whose length is no multiple of 8, two taps at a time (Th2 is even): window
+            // elements 15 - (a0 mod 16) ... of the block, padded from the 16th on (6 taps per plane, 2^16 samples:
+            // 38.9 -> 35.8 us a call). With fewer planes the loop below stays: their blocks of 16 come out slower
+            // beside this one (decimation 8, 32 taps per plane, 2^24 samples: 203.5 -> 204.8 us)
+            for (; a0 < Th2; a0 += 2) {
+                const int k0 = 15 - (a0 & 15);
+                float x[kDdcPer + 1];
+#pragma unroll
+                for (int i = 0; i <= kDdcPer; i++) x[i] = w[k0 + i + (k0 + i >= 16 ? 1 : 0)];
+                const float4 two = *reinterpret_cast<const float4 *>(h + a0);
+#pragma unroll
+                for (int r = 0; r < kDdcPer; r++)
+                    acc[r] = __ffma2_rn(make_float2(two.x, two.y), make_float2(x[r + 1], x[r + 1]), acc[r]);
+#pragma unroll
+                for (int r = 0; r < kDdcPer; r++)
+                    acc[r] = __ffma2_rn(make_float2(two.z, two.w), make_float2(x[r], x[r]), acc[r]);
+            }
+        } else {
+            for (int a = a0; a < Th2; a++) {   // taps left over when Th2 is not a multiple of 8
+                const float2 ha = h[a];
+                const int base = kDdcPer * t + Th2 + shift - a;
+#pragma unroll
+                for (int r = 0; r < kDdcPer; r++) {
+                    const float x = plane[ppos(base + r)];
+                    acc[r] = __ffma2_rn(ha, make_float2(x, x), acc[r]);
+                }
+            }
         }
     }
     // rotation exp(2 pi i (j / 4 - fc i0)), i0 = j D2: the first output's
