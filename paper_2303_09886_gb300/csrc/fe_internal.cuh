@@ -302,6 +302,7 @@ struct Phase1TcParams {
     int *err;                 // set to 2 if a bounded wait gave up
 };
 int phase1_tc_R(int N);
+bool phase1_tc_streamed(int N);
 int phase1_tc_layout(int N, int precision);   // layout of the intermediate that phase 1 writes
 bool phase1_tc_supported(int N, int T, int precision);
 int phase1_tc_phys(int N, int T, int precision);
@@ -309,12 +310,14 @@ void build_phase1_tc_tables(int N, int T, int precision, const float *w, std::ve
                             std::vector<float> &oscale, float &s_int);
 cudaError_t launch_phase1_tc(int T, int precision, const Phase1TcParams &p, cudaStream_t s, bool pdl);
 cudaError_t launch_unpack_cols(const UnpackColsParams &p, cudaStream_t s, bool pdl);
-// rows of the FP16 column buffer: a call's history + chunk plus the reach of
-// a 128-spectrum pass past the chunk end, padded to a multiple of 64
+// rows of the FP16 column buffer: a call's history + chunk, and what the copies
+// reach past them (k_phase1_tc: a whole 128-spectrum pass; k_phase1_ts: its
+// runs' own rows, the padded single tap, the realigned copy's extra chunk), a
+// multiple of 64
 inline int unpack_cols_rows(long long H, long long L, long long D, long long Dmin, int N, int T) {
     const long long P = N / 8;
     const long long rt = (H + L + D - Dmin) / P + 3 + 8;
-    const long long reach = 8LL * (127 + (T < 2 ? 2 : T)) + 64;
+    const long long reach = phase1_tc_streamed(N) ? 64 : 8LL * (127 + (T < 2 ? 2 : T)) + 64;
     return (int)((rt + reach + 63) / 64 * 64);
 }
 

@@ -825,6 +825,13 @@ __global__ void __launch_bounds__(tc_threads(tc_one_cta(PH, R, T, PREC)), tc_one
 // two columns between the lanes of a spectrum pair and stores the second
 // stage's pairs, 16 bytes (FP16: 8) per lane.
 //
+// A run's copies bring the rows that it reads and no others, and where columns
+// wrap (the first or last few of a unit, at a delay other than the columns'
+// own) only those are realigned: 64 spectra of 32768 channels, FP16, a delay
+// step every 5 spectra, 1299 -> 1045 us a call, every 33, 273 -> 236. (Steps as
+// dense as the first are the one shape that the resident blocks of k_phase1_tc
+// took better, 770 us: every run streams the blocks once more.)
+//
 // What bounds it: with one lane running the MMA loop, its issue (0.557 ms ->
 // 0.36 at R = 4 in FP16); since the whole warp runs it and one elected lane
 // issues, an MMA (128 x 80 x 16 at R = 8) takes 127 cycles, of which the
@@ -1004,15 +1011,8 @@ __global__ void __launch_bounds__(kTsThreads, 1) k_phase1_ts(const __grid_consta
         }
         for (;;) {
             int nact = 0;          // tiles with a run in this round
-            bool moved = p.window_tap != nullptr;   // a run that reads other rows than the columns' own delay
 #pragma unroll
-            for (int g = 0; g < G; g++) {
-                const bool act = tl[g].ra < tl[g].rows;
-                nact += act ? 1 : 0;
-                // a run at another delay reads other columns of the same rows, where none of the unit's wraps
-                const int dc = tl[g].c0 - tl[g].c;
-                moved = moved || (act && (dc + t2 < 0 || dc + t2 + CW > N2));
-            }
+            for (int g = 0; g < G; g++) nact += tl[g].ra < tl[g].rows ? 1 : 0;
             if (nact == 0 || !ok) break;
             if (warp >= 4 && warp < 8) {
                 // ---------------- fill ----------------
@@ -1026,96 +1026,152 @@ __global__ void __launch_bounds__(kTsThreads, 1) k_phase1_ts(const __grid_consta
                                  : "memory");
                     return go != 0;
                 };
-                auto copy = [&]() -> bool {
+                // physical column that tile ps reads for step cj: t + c0 - c (the columns are laid out at delay
+                // c0). One of them starts at row 8 (m0 + q0) - rb, 16-byte aligned, and takes one bulk copy per
+                // plane; what wraps into the row before or after is realigned
+                auto column = [&](const TsTile &ps, int cj) -> int {
+                    constexpr int far = 1 << 20;   // (past every column)
+                    return max(-far, min(far, ps.c0 - ps.c)) + t2 + cj / R + N2 * (cj % R);
+                };
+                auto wraps = [&](const TsTile &ps, int cj) -> bool {
+                    const int t = column(ps, cj);
+                    return t < 0 || t >= P || p.window_tap;   // (the debug tap is read where the realigned copy is)
+                };
+                // only what the run's rows read (the rest of the tile is left as it is: a row of the accumulator
+                // depends on its own row alone)
+                auto run_bytes = [&](const TsTile &ps) -> uint32_t { return 16u * (uint32_t)(ps.rb - ps.ra + TP - 1); };
+                auto first_row = [&](const TsTile &ps) -> long long { return 8LL * (p.m0 + ps.q0 + ps.ra) - p.rb; };
+                bool any = false;   // (the first and the last column are the outermost steps)
+#pragma unroll
+                for (int g = 0; g < G; g++)
+                    any = any || (tl[g].ra < tl[g].rows && (wraps(tl[g], 0) || wraps(tl[g], CW * R - 1)));
+                auto stage_free = [&](int k) -> bool {
+                    const unsigned n = ns + (unsigned)k;
+                    return n < NS || wait_bar(&empty[n % NS], ((n / NS) - 1) & 1);
+                };
+                auto copy = [&]() -> bool {   // each warp its own tile, one lane
                     bool go = true;
-                    // a sequence starts at row 8 (m0 + q0) - rb, 16-byte aligned, of column t + c0 - c (the
-                    // columns are laid out at delay c0); one bulk copy per plane, each warp its own tile
 #pragma unroll
                     for (int g = 0; g < G; g++) {
                         if (warp != 4 + g || lane != 0) continue;
                         const TsTile &ps = tl[g];
                         const bool act = ps.ra < ps.rows;
-                        const uint16_t *col =
-                            p.cols + ((long long)ps.st * P + t2 + (ps.c0 - ps.c)) * p.RTP + (8LL * (p.m0 + ps.q0) - p.rb);
-                        for (int k = 0; k < NST && go; k++) {
-                            const unsigned n = ns + (unsigned)k, s = n % NS;
-                            go = n < NS || wait_bar(&empty[s], ((n / NS) - 1) & 1);
+                        const uint16_t *col = p.cols + ((long long)ps.st * P + column(ps, 0)) * p.RTP + first_row(ps);
+                        const uint32_t bytes = run_bytes(ps);
+                        for (int k = 0; k < NST; k++) {
+                            const unsigned s = (ns + (unsigned)k) % NS;
+                            uint8_t *xb = smem + s * ST + SJ * BB + g * AB + 16 * ps.ra;
+                            const uint16_t *src[SJ];
+#pragma unroll
+                            for (int i = 0; i < SJ; i++)
+                                src[i] = col + (long long)((k * SJ + i) / R + N2 * ((k * SJ + i) % R)) * p.RTP;
+                            // (addresses before the wait: what lies between a stage's release and its copies is
+                            // time that the stage stands empty; 32768 channels, FP16, 256 spectra of two streams:
+                            // 169 -> 156 us)
+#pragma unroll
+                            for (int i = 0; i < SJ; i++) asm volatile("" ::"l"(src[i]));
+                            if (go) go = stage_free(k);
                             if (!go) break;
                             if (!act) {
                                 arrive(&full[s]);
                                 continue;
                             }
-                            expect(&full[s], SJ * AB);
+                            expect(&full[s], SJ * NPL * bytes);
 #pragma unroll
-                            for (int i = 0; i < SJ; i++) {
-                                const int cj = k * SJ + i;
-                                const uint16_t *src = col + (long long)(cj / R + N2 * (cj % R)) * p.RTP;
-                                uint8_t *xb = smem + s * ST + SJ * BB + (i * G + g) * AB;
+                            for (int i = 0; i < SJ; i++)
 #pragma unroll
                                 for (int pl = 0; pl < NPL; pl++)
-                                    bulk(xb + pl * XL * 2, src + pl * p.plane_elems, XL * 2, &full[s]);
-                            }
+                                    bulk(xb + i * G * AB + pl * XL * 2, src[i] + pl * p.plane_elems, bytes, &full[s]);
                         }
                     }
                     __syncwarp();
                     return __shfl_sync(0xFFFFFFFFu, (int)go, 0) != 0;
                 };
-                auto stage_free = [&](int k) -> bool {
-                    const unsigned n = ns + (unsigned)k;
-                    return ft != 0 || n < NS || wait_bar(&empty[n % NS], ((n / NS) - 1) & 1);
-                };
                 auto realign = [&](int k) {
                     const unsigned s = (ns + (unsigned)k) % NS;
-#pragma unroll 1
-                    for (int i = 0; i < SJ; i++) {
-                        const int c = (k * SJ + i) / R, j = (k * SJ + i) % R;
-                        const long long t = t2 + c + (long long)N2 * j;   // physical column
+                    // the steps that do not wrap, counted without an arrival (that follows below)
 #pragma unroll
-                        for (int g = 0; g < G; g++) {
-                            const TsTile &ps = tl[g];
-                            if (ps.ra >= ps.rows) continue;
-                            uint8_t *xb = smem + s * ST + SJ * BB + (i * G + g) * AB;
-                            // 16-byte chunks from the aligned element row0 - sh, each output chunk 16 bytes
-                            // at byte offset 2 sh of two consecutive source chunks
-                            const long long a0 = (long long)p.N * (p.m0 + ps.q0) - ps.c + ps.c0 + t;
-                            const long long ra = floor_div(a0, P);
-                            const long long row0 = ra - p.rb;
-                            const uint16_t *src =
-                                p.cols + ((long long)ps.st * P + (a0 - ra * P)) * p.RTP + (row0 & ~7LL);
-                            const int sh = (int)(row0 & 7);
-                            constexpr int CPC = XL / 8;
-                            for (int e = ft; e < NPL * CPC; e += kTsFill) {
-                                const int pl = e / CPC, q8 = e - pl * CPC;
-                                const uint4 *q = reinterpret_cast<const uint4 *>(src + pl * p.plane_elems) + q8;
-                                const uint4 v0 = ld_dep(q), v1 = ld_dep(q + 1);
-                                const uint32_t w[8] = {v0.x, v0.y, v0.z, v0.w, v1.x, v1.y, v1.z, v1.w};
-                                const uint32_t sel = (sh & 1) ? 0x5432u : 0x3210u;   // 2-byte shift for odd sh
-                                uint32_t o[4];
+                    for (int g = 0; g < G; g++) {
+                        if (warp != 4 + g || lane != 0 || tl[g].ra >= tl[g].rows) continue;
 #pragma unroll
-                                for (int m = 0; m < 4; m++) {
-                                    uint32_t lo = w[m], hi = w[m + 1];
-                                    if ((sh >> 1) == 1) lo = w[m + 1], hi = w[m + 2];
-                                    else if ((sh >> 1) == 2) lo = w[m + 2], hi = w[m + 3];
-                                    else if ((sh >> 1) == 3) lo = w[m + 3], hi = w[m + 4];
-                                    o[m] = __byte_perm(lo, hi, sel);
-                                }
-                                reinterpret_cast<uint4 *>(xb + pl * XL * 2)[q8] = make_uint4(o[0], o[1], o[2], o[3]);
+                        for (int i = 0; i < SJ; i++)
+                            if (!wraps(tl[g], k * SJ + i)) {
+                                asm volatile("mbarrier.expect_tx.relaxed.cta.shared::cta.b64 [%0], %1;" ::"r"(
+                                                 smem_addr(&full[s])),
+                                             "r"(NPL * run_bytes(tl[g]))
+                                             : "memory");
+                                const uint16_t *src =
+                                    p.cols + ((long long)tl[g].st * P + column(tl[g], k * SJ + i)) * p.RTP + first_row(tl[g]);
+                                uint8_t *xb = smem + s * ST + SJ * BB + (i * G + g) * AB + 16 * tl[g].ra;
+#pragma unroll
+                                for (int pl = 0; pl < NPL; pl++)
+                                    bulk(xb + pl * XL * 2, src + pl * p.plane_elems, run_bytes(tl[g]), &full[s]);
                             }
-                            if (p.window_tap) {
-                                // debug tap: the first FIR tap of spectrum q0 + v / 8 at offset P (v % 8) + t
-                                asm volatile("bar.sync 1, %0;" ::"n"(kTsFill) : "memory");
-                                const uint16_t *xv = reinterpret_cast<const uint16_t *>(xb);
-                                for (int vv = ft; vv < 8 * kTcRows; vv += kTsFill) {
-                                    const int mrow = vv >> 3;
-                                    if (mrow < ps.ra || mrow >= ps.rb) continue;
-                                    float x;
-                                    if constexpr (PREC == 2)
-                                        x = __bfloat162float(__ushort_as_bfloat16(xv[vv])) +
-                                            __bfloat162float(__ushort_as_bfloat16(xv[XL + vv]));
-                                    else x = __half2float(__ushort_as_half(xv[vv]));
-                                    p.window_tap[((long long)ps.st * p.M + ps.q0 + mrow) * p.N +
-                                                 (long long)P * (vv & 7) + t] = (int)x;
-                                }
+                    }
+                    __syncwarp();
+#pragma unroll 1
+                    for (int x = 0; x < SJ * G; x++) {
+                        const int i = x / G, g = x % G, cj = k * SJ + i;
+                        TsTile ps;   // tl[g] (registers: selected by comparison)
+#pragma unroll
+                        for (int y = 0; y < G; y++)
+                            if (y == g) ps = tl[y];
+                        if (ps.ra >= ps.rows || !wraps(ps, cj)) continue;
+                        const long long t = t2 + cj / R + (long long)N2 * (cj % R);   // physical column
+                        uint8_t *xb = smem + s * ST + SJ * BB + (i * G + g) * AB;
+                        // 16-byte chunks from the aligned element row0 - sh, each output chunk 16 bytes
+                        // at byte offset 2 sh of two consecutive source chunks; a thread's loads together
+                        const long long a0 = (long long)p.N * (p.m0 + ps.q0) - ps.c + ps.c0 + t;
+                        const long long ra = floor_div(a0, P);
+                        const long long row0 = ra - p.rb;
+                        const uint16_t *src = p.cols + ((long long)ps.st * P + (a0 - ra * P)) * p.RTP + (row0 & ~7LL);
+                        const int sh = (int)(row0 & 7);
+                        const uint32_t sel = (sh & 1) ? 0x5432u : 0x3210u;   // 2-byte shift for odd sh
+                        constexpr int NIT = (NPL * (XL / 8) + kTsFill - 1) / kTsFill;
+                        const int cpc = ps.rb - ps.ra + TP - 1;   // chunks of the run, per plane
+                        uint4 v[NIT][2];
+#pragma unroll
+                        for (int it = 0; it < NIT; it++) {
+                            const int e = ft + it * kTsFill;
+                            if (e >= NPL * cpc) continue;
+                            const int pl = NPL > 1 && e >= cpc;
+                            const uint4 *q = reinterpret_cast<const uint4 *>(src + pl * p.plane_elems) + ps.ra + e - pl * cpc;
+                            v[it][0] = ld_dep(q);
+                            v[it][1] = ld_dep(q + 1);
+                        }
+#pragma unroll
+                        for (int it = 0; it < NIT; it++) {
+                            const int e = ft + it * kTsFill;
+                            if (e >= NPL * cpc) continue;
+                            const int pl = NPL > 1 && e >= cpc;
+                            const uint4 v0 = v[it][0], v1 = v[it][1];
+                            const uint32_t w[8] = {v0.x, v0.y, v0.z, v0.w, v1.x, v1.y, v1.z, v1.w};
+                            uint32_t o[4];
+#pragma unroll
+                            for (int m = 0; m < 4; m++) {
+                                uint32_t lo = w[m], hi = w[m + 1];
+                                if ((sh >> 1) == 1) lo = w[m + 1], hi = w[m + 2];
+                                else if ((sh >> 1) == 2) lo = w[m + 2], hi = w[m + 3];
+                                else if ((sh >> 1) == 3) lo = w[m + 3], hi = w[m + 4];
+                                o[m] = __byte_perm(lo, hi, sel);
+                            }
+                            reinterpret_cast<uint4 *>(xb + pl * XL * 2)[ps.ra + e - pl * cpc] =
+                                make_uint4(o[0], o[1], o[2], o[3]);
+                        }
+                        if (p.window_tap) {
+                            // debug tap: the first FIR tap of spectrum q0 + v / 8 at offset P (v % 8) + t
+                            asm volatile("bar.sync 1, %0;" ::"n"(kTsFill) : "memory");
+                            const uint16_t *xv = reinterpret_cast<const uint16_t *>(xb);
+                            for (int vv = ft; vv < 8 * kTcRows; vv += kTsFill) {
+                                const int mrow = vv >> 3;
+                                if (mrow < ps.ra || mrow >= ps.rb) continue;
+                                float x;
+                                if constexpr (PREC == 2)
+                                    x = __bfloat162float(__ushort_as_bfloat16(xv[vv])) +
+                                        __bfloat162float(__ushort_as_bfloat16(xv[XL + vv]));
+                                else x = __half2float(__ushort_as_half(xv[vv]));
+                                p.window_tap[((long long)ps.st * p.M + ps.q0 + mrow) * p.N +
+                                             (long long)P * (vv & 7) + t] = (int)x;
                             }
                         }
                     }
@@ -1123,7 +1179,7 @@ __global__ void __launch_bounds__(kTsThreads, 1) k_phase1_ts(const __grid_consta
                     asm volatile("bar.sync 1, %0;" ::"n"(kTsFill) : "memory");
                     if (lane == 0 && warp < 4 + G) arrive(&full[s]);
                 };
-                ok = ts_fill_round<NST>(moved, copy, stage_free, realign, vote);
+                ok = ts_fill_round<NST>(any, copy, [&](int k) { return ft != 0 || stage_free(k); }, realign, vote);
             } else if (warp == 9) {
                 // ---------------- operand blocks ----------------
                 if (lane == 0) {
