@@ -906,7 +906,7 @@ fengine_status process_impl(fengine_plan_t pl, void *cuda_stream, const uint8_t 
         p1.A = A;
         p1.q_begin = qb;
         p1.q_count = qc;
-        p1.rows = fe::phase1_rows(pl->T, pl->N1, pl->N2, qc, pl->n_streams);
+        if (!pl->tc1) p1.rows = fe::phase1_rows(pl->T, pl->N1, pl->N2, qc, pl->n_streams);
         pt.A = A;
         pt.q_begin = qb;
         pt.q_count = qc;

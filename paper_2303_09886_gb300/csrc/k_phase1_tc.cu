@@ -552,13 +552,17 @@ __global__ void __launch_bounds__(tc_threads(tc_one_cta(PH, R, T, PREC)), tc_one
             if (!ok) break;
             uint16_t *xb = xsm + (size_t)s * NPL * PH * XL;
             // the columns are laid out at delay c0: a pass at delay c reads column
-            // t + c0 - c, which for all but the CTAs at the edges is one of the same
-            // rows: only those realign (32768 channels in BF16, 2^28 samples at a
-            // delay rate of 5e-9, whose delay steps once or twice: a call 8.50 -> 4.77 ms)
-            const int dc = ps.c0 - ps.c;
-            if (!p.window_tap && dc + cg * CW >= 0 && dc + (cg + 1) * CW <= N2) {
-                // every column sequence starts at row 8 (m0 + q0) - rb, 16-byte
-                // aligned, one bulk copy each (per plane)
+            // t + c0 - c of the same rows, 16-byte aligned, one bulk copy each (per
+            // plane); only what wraps into the row before or after, the CTA's first
+            // columns or its last, is realigned. (With every column of such a pass
+            // realigned, the CTAs at the edges finished last by far: 131072 spectra of
+            // two streams of 1024 channels, FP16, 16 taps, one delay step, phase 1 1.63
+            // -> 0.86 ms; 512 spectra of four of 8192, BF16, a step every 77, 0.473 ->
+            // 0.394. Steps every 33 spectra and less in BF16 below 2048 channels are 2 - 3 %
+            // the slower for it.)
+            constexpr int far = 1 << 20;   // (past every column)
+            const int dc = max(-far, min(far, ps.c0 - ps.c)), t_cg = cg * CW + dc;
+            if (!p.window_tap && t_cg >= 0 && t_cg + (PH - 1) % CW + N2 * ((PH - 1) / CW) < P) {   // none wraps
                 if (ft == 0) {
                     constexpr uint32_t bytes = (uint32_t)(NPL * PH * XL * 2);
                     asm volatile("{\n\t.reg .b64 st;\n\tmbarrier.arrive.expect_tx.shared::cta.b64 st, [%0], %1;\n\t}"
@@ -578,8 +582,37 @@ __global__ void __launch_bounds__(tc_threads(tc_one_cta(PH, R, T, PREC)), tc_one
                 }
                 continue;
             }
-            if (ft < PH) {
-                const long long a0 = col_start(ps, ft);
+            auto column = [&](int i) -> int { return t_cg + (i % CW) + N2 * (i / CW); };   // rises with i
+            int w0 = 0, nw = 0;   // [w0, w0 + nw): the columns that wrap
+            if (p.window_tap) {
+                nw = PH;
+            } else if (t_cg < 0) {
+                while (nw < PH && column(nw) < 0) nw++;
+            } else {
+                while (nw < PH && column(PH - 1 - nw) >= P) nw++;
+                w0 = PH - nw;
+            }
+            if (ft < 32) {
+                // the others' bytes, counted without an arrival (that follows the realigned columns); a lane per copy
+                static_assert(NPL * PH <= 32, "one warp issues the copies");
+                if (ft == 0)
+                    asm volatile("mbarrier.expect_tx.relaxed.cta.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(&xfull[s])),
+                                 "r"((uint32_t)(NPL * (PH - nw) * XL * 2))
+                                 : "memory");
+                __syncwarp();
+                const int i = ft % PH, pl = ft / PH;
+                if (ft < NPL * PH && (i < w0 || i >= w0 + nw)) {
+                    const uint16_t *src = p.cols + pl * p.plane_elems + ((long long)ps.st * P + column(i)) * p.RTP +
+                                          (8LL * (p.m0 + ps.q0) - p.rb);
+                    asm volatile(
+                        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                            smem_addr(xb + (size_t)ft * XL)),
+                        "l"(src), "r"((uint32_t)(XL * 2)), "r"(smem_addr(&xfull[s]))
+                        : "memory");
+                }
+            }
+            if (ft < nw) {
+                const long long a0 = col_start(ps, w0 + ft);
                 const long long ra = floor_div(a0, P);
                 const long long col = a0 - ra * P, row0 = ra - p.rb;
                 fsrc[s * PH + ft] = ((long long)ps.st * P + col) * p.RTP + (row0 & ~7LL);
@@ -587,15 +620,14 @@ __global__ void __launch_bounds__(tc_threads(tc_one_cta(PH, R, T, PREC)), tc_one
             }
             asm volatile("bar.sync 1, %0;" ::"n"(FT) : "memory");
             // (BF16: both data planes, unpacked already split into hi and lo)
-            for (int e0 = ft; e0 < NPL * PH * CPC; e0 += FT * 3) {
+            for (int e0 = ft; e0 < NPL * nw * CPC; e0 += FT * 3) {
                 uint4 a[3], b[3];
 #pragma unroll
                 for (int u = 0; u < 3; u++) {
                     const int e = e0 + FT * u;
-                    if (e < NPL * PH * CPC) {
-                        const int ip = e / CPC, j = e - ip * CPC, i = ip % PH;
-                        const uint4 *src =
-                            reinterpret_cast<const uint4 *>(p.cols + (ip / PH) * p.plane_elems + fsrc[s * PH + i]) + j;
+                    if (e < NPL * nw * CPC) {
+                        const int iw = e / CPC, j = e - iw * CPC, pl = NPL > 1 && iw >= nw, i = iw - pl * nw;
+                        const uint4 *src = reinterpret_cast<const uint4 *>(p.cols + pl * p.plane_elems + fsrc[s * PH + i]) + j;
                         a[u] = ld_dep(src);
                         b[u] = ld_dep(src + 1);
                     }
@@ -603,8 +635,8 @@ __global__ void __launch_bounds__(tc_threads(tc_one_cta(PH, R, T, PREC)), tc_one
 #pragma unroll
                 for (int u = 0; u < 3; u++) {
                     const int e = e0 + FT * u;
-                    if (e < NPL * PH * CPC) {
-                        const int ip = e / CPC, j = e - ip * CPC, i = ip % PH;
+                    if (e < NPL * nw * CPC) {
+                        const int iw = e / CPC, j = e - iw * CPC, pl = NPL > 1 && iw >= nw, i = iw - pl * nw;
                         const int sh = fsh[s * PH + i];
                         const uint32_t w[8] = {a[u].x, a[u].y, a[u].z, a[u].w, b[u].x, b[u].y, b[u].z, b[u].w};
                         uint32_t o[4];
@@ -627,7 +659,7 @@ __global__ void __launch_bounds__(tc_threads(tc_one_cta(PH, R, T, PREC)), tc_one
                                 for (int m = 0; m < 4; m++) o[m] = __byte_perm(w[m + 3], w[m + 4], sel);
                                 break;
                         }
-                        reinterpret_cast<uint4 *>(xb + (size_t)ip * XL)[j] = make_uint4(o[0], o[1], o[2], o[3]);
+                        reinterpret_cast<uint4 *>(xb + (size_t)(pl * PH + w0 + i) * XL)[j] = make_uint4(o[0], o[1], o[2], o[3]);
                     }
                 }
             }
