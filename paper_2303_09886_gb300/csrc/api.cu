@@ -45,7 +45,7 @@ long long coarse_delay(const DelaySeg &s, long long t0) {
 
 struct fengine_plan_s {
     int device = 0;
-    int n_ant = 0, n_streams = 0, n = 0, N = 0, T = 0, S = 0, M = 0, N1 = 0, N2 = 0, W = 0, C = 0, R2 = 0;
+    int n_ant = 0, n_streams = 0, n = 0, N = 0, T = 0, S = 0, M = 0, N1 = 0, N2 = 0, W = 0, R2 = 0;
     int precision = 0;
     int a_elem = 8;                 // bytes per intermediate element
     long long L = 0, D = 0, Dmin = 0, H = 0, chunk_bytes = 0, hist_bytes = 0;
@@ -306,7 +306,6 @@ fengine_status fengine_plan_create(const fengine_config *cfg, fengine_plan_t *ou
     pl->tc1 = tc1;
     pl->N2 = (int)(N / pl->N1);
     pl->W = fe::phase1_W(pl->N1, pl->N2);
-    pl->C = pl->N1 * pl->W;
     pl->R2 = fe::phase2_R2(pl->N2);
     // the history reaches back to the earliest window start of the call's
     // first spectrum: N (T - 1 + E) + D samples before the chunk
@@ -741,7 +740,6 @@ fengine_status process_impl(fengine_plan_t pl, void *cuda_stream, const uint8_t 
     p1.N = pl->N;
     p1.N2 = pl->N2;
     p1.W = pl->W;
-    p1.C = pl->C;
     p1.M = pl->M;
     p1.m0 = m0;
     p1.t_in = first_sample;
@@ -976,7 +974,7 @@ fengine_status fengine_device_status(fengine_plan_t pl) {
     if ((e = cudaMemcpy(&h, pl->d_err, sizeof(int), cudaMemcpyDeviceToHost)) != cudaSuccess ||
         (e = cudaMemset(pl->d_err, 0, sizeof(int))) != cudaSuccess)
         return cuda_fail(e, "device status");
-    if (h == 2) return fail(FENGINE_ETIMEOUT, "a bounded wait of the tensor-core phase 1 gave up");
+    if (h == 2) return fail(FENGINE_ETIMEOUT, "a bounded wait of a kernel gave up (tensor-core phase 1, or a copy of the second stage)");
     if (h == 1) return fail(FENGINE_EDELAY, "a coarse delay was clamped on the device");
     return FENGINE_OK;
 }

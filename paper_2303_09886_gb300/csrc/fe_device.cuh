@@ -1,5 +1,5 @@
 // Device helpers shared by the libfengine kernels: complex arithmetic, the
-// 10-bit sample fetch, the quantiser and an in-register radix-2 FFT.
+// quantiser and an in-register radix-2 FFT.
 #pragma once
 #include <cstdint>
 #include <cuda_runtime.h>
@@ -12,21 +12,6 @@ __host__ __device__ __forceinline__ float2 cmul(float2 a, float2 b) {
     return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }
 __host__ __device__ __forceinline__ float2 cconj(float2 a) { return make_float2(a.x, -a.y); }
-// The same sums as packed FP32x2 instructions (two round-to-nearest adds in
-// one; the results are those of cadd and csub).
-__device__ __forceinline__ float2 cadd2(float2 a, float2 b) { return __fadd2_rn(a, b); }
-__device__ __forceinline__ float2 csub2(float2 a, float2 b) { return __fadd2_rn(a, make_float2(-b.x, -b.y)); }
-
-// Sample j of a packed 10-bit stream (bits [10 j, 10 j + 10), most
-// significant bit first, two's complement; Sec. 2.2 fixes 10 bits/sample).
-// The field lies in bytes 5j/4 and 5j/4 + 1 at bit offset 2 (j mod 4).
-__device__ __forceinline__ int fetch10(const uint8_t *__restrict__ p, long long j) {
-    const long long byte = (5 * j) >> 2;
-    const int r = 2 * (int)(j & 3);
-    unsigned v = ((unsigned)__ldg(p + byte) << 8) | (unsigned)__ldg(p + byte + 1);
-    v = (v >> (6 - r)) & 0x3FFu;
-    return (int)v - (int)((v & 0x200u) << 1);
-}
 
 // Requantise to an 8-bit Gaussian-integer component (Sec. 2.1 step 6,
 // Sec. 3.6): saturate to [-127, 127], round half away from zero. Adding the
@@ -34,7 +19,7 @@ __device__ __forceinline__ int fetch10(const uint8_t *__restrict__ p, long long 
 // from zero and everything else to nearest for |t| <= 127 (FP32 addition is
 // correctly rounded, so t + 0.49999997 reaches the next integer exactly when
 // frac(|t|) >= 1/2). This is the rule on the host; the kernels apply it to
-// four components at a time (quant8x4).
+// four components at a time, with other steps (quant8x4).
 inline int quant8(float x) {
     const float t = fminf(fmaxf(x, -127.0f), 127.0f);
     return (int)(t + copysignf(0.49999997f, t));

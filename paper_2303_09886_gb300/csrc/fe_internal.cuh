@@ -8,12 +8,14 @@
 //   k_phase2w       1024-point FFT over t2 + fine-delay rotation + gain +
 //                   requantise + channel-major corner turn (persistent, one
 //                   warp per pair of spectra), or
-//   k_phase2<N2>    the same for N2 < 1024
-// In the reduced-precision forms phase 1 is k_phase1_tc (tcgen05 tensor
-// cores: unpack + coarse delay + FIR + first DFT stage with its twiddle in one
-// contraction); the second stage reads its FP16 (FP16 form) or FP32 (BF16
-// form) output.
-// with the four-step split t = N2 t1 + t2, k = k1 + N1 k2 of the 2n-point
+//   k_phase2_pairs  the same for N2 = 512, and for large calls of N2 = 256
+//   k_phase2<N2>    the same for smaller N2 and small calls of N2 = 256
+// In the reduced-precision forms k_unpack_cols writes the samples as 16-bit
+// columns, and phase 1 is k_phase1_tc or, from 16384 channels, k_phase1_ts
+// (tcgen05 tensor cores: coarse delay + FIR + first DFT stage with its twiddle
+// in one contraction); the second stage reads its FP16 (FP16 form) or FP32
+// (BF16 form) output.
+// All with the four-step split t = N2 t1 + t2, k = k1 + N1 k2 of the 2n-point
 // real DFT (the exp(-2 pi i k1 t2 / N) cross term is the twiddle).
 #pragma once
 #include <cstddef>
@@ -66,7 +68,6 @@ struct LostDataParams {
     int HV;                          // history heaps kept
     long long heap0;                 // t_in / kHeapSamples
     int chunk_heaps;                 // L / kHeapSamples
-    const int *ctab;                 // [stream][M]
     int n_ant, N, T, M, S;
     long long m0;
     unsigned char *heap_flags;       // out [ant][ceil(M / S)], nullptr = not wanted
@@ -77,16 +78,15 @@ struct Phase1Params {
     long long chunk_bytes, hist_bytes;
     long long H;              // history samples (multiple of 4)
     long long L;              // chunk samples
-    int N, N2, W, C;          // FFT length, second-stage size, t2 per CTA, columns per CTA
+    int N, N2, W;             // FFT length, second-stage size, t2 per CTA
     int M;                    // spectra per call
     long long m0;             // first spectrum of the call
     long long t_in;           // first sample of the chunk
     const float *w;           // [N*T] prototype, w[t + N j]
     const float2 *tw1;        // [(N1/2+1)][N2] exp(-2 pi i k1 t2 / N)
     const int *ctab;          // [stream][M]
-    float2 *A;                // out, spectrum q at row q - q_begin: N1 <= 32 in spectrum pairs,
-                              // [stream][a_spectra / 2][N1/2+1][N2] of (re, re, im, im), else
-                              // [stream][a_spectra][N1/2+1][N2] of (re, im)
+    float2 *A;                // out, spectrum q at row q - q_begin, in spectrum pairs:
+                              // [stream][a_spectra / 2][N1/2+1][N2] of (re, re, im, im)
     int rows;                 // spectra per CTA: even, at most kP1Blocks * kP1Block
     int *window_tap;          // optional out [stream][M][N]
     int q_begin, q_count;     // the slab of spectra this launch covers
@@ -111,7 +111,7 @@ struct Phase2Params {
     int N, N1, M, S, R2;      // FFT length, first-stage size, spectra/call, spectra/heap, spectra/CTA
     int8_t *out;              // [ant][heap][n][S_h][pol][2]
     float2 *prequant;         // optional [stream][M][n]
-    int in;                   // layout of A: kInPairs, kInHalf or kInFloat
+    int in;                   // layout of A: kInPairs, kInHalf, kInFloat or kInHalfPairs
     int *err;                 // set to 2 if a bounded wait gave up (may be nullptr)
     float tc_unscale;         // inverse of the power-of-two scale of an FP16 A (1 otherwise)
 };

@@ -506,29 +506,30 @@ int phase2_blocks(int N2, const Phase2Params &p, int n_ant, int *gx, int *gy) {
 // (g = nullptr: only the kernel's shared-memory size is set)
 template <int N2, int IN, int CAP>
 static cudaError_t launch_p2(const GroupArgs<Phase2Params, CAP> *g, cudaStream_t s, bool pdl) {
-    const int R2 = P2Shape<N2>::R2;
-    void (*kernel)(GroupArgs<Phase2Params, CAP>) = k_phase2<N2, IN, CAP>;
-    size_t smem = phase2_smem_bytes(N2, R2);
-    unsigned threads = kP2Threads;
-    if (!g) {
-        const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if constexpr (N2 >= 256) {
-            if (e == cudaSuccess)
-                return cudaFuncSetAttribute(k_phase2_pairs<N2, IN, CAP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                            (int)sizeof(typename P2Pair<N2>::Smem));
-        }
-        return e;
-    }
+    constexpr int R2 = phase2_R2_for(N2);
+    void (*kernel)(GroupArgs<Phase2Params, CAP>) = nullptr;
+    size_t smem = 0;
+    unsigned threads = 0;
+    // On pairs from where it is the faster: N2 = 512 always (8 taps, one antenna: 16 spectra 11.8 against
+    // 12.8 us, 16384 spectra 0.322 against 0.390 ms), N2 = 256 from two waves of its CTAs on (2048 spectra
+    // 24.5 against 26.6 us, 16384 0.145 against 0.165 ms; 16 spectra 9.8 against 8.7 us, where half the
+    // threads per spectrum make a CTA's chain longer and nothing else runs beside it)
     if constexpr (N2 >= 256) {
-        // On pairs from where it is the faster: N2 = 512 always (8 taps, one antenna: 16 spectra 11.8 against
-        // 12.8 us, 16384 spectra 0.322 against 0.390 ms), N2 = 256 from two waves of its CTAs on (2048 spectra
-        // 24.5 against 26.6 us, 16384 0.145 against 0.165 ms; 16 spectra 9.8 against 8.7 us, where half the
-        // threads per spectrum make a CTA's chain longer and nothing else runs beside it)
-        if (N2 == 512 || g->start[g->n] >= 8 * phase2w_wave()) {
-            kernel = k_phase2_pairs<N2, IN, CAP>;
-            smem = sizeof(typename P2Pair<N2>::Smem);
-            threads = P2Pair<N2>::THREADS;
+        kernel = k_phase2_pairs<N2, IN, CAP>;
+        smem = sizeof(typename P2Pair<N2>::Smem);
+        threads = P2Pair<N2>::THREADS;
+        if (!g) {
+            const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            if (e != cudaSuccess || N2 == 512) return e;
         }
+    }
+    if constexpr (N2 != 512) {
+        if (N2 < 256 || !g || g->start[g->n] < 8 * phase2w_wave()) {
+            kernel = k_phase2<N2, IN, CAP>;
+            smem = phase2_smem_bytes(N2, R2);
+            threads = kP2Threads;
+        }
+        if (!g) return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     }
     for (int m = 0; m < g->n; m++)
         if (g->p[m].R2 != R2 || g->p[m].a_spectra % 2) return cudaErrorInvalidValue;

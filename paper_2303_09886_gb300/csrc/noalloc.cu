@@ -202,7 +202,6 @@ fengine_status fengine_process_chunk_noalloc(const fengine_noalloc_args *a, cons
     p1.N = (int)N;
     p1.N2 = N2;
     p1.W = fe::phase1_W(N1, N2);
-    p1.C = N1 * p1.W;
     p1.M = (int)M;
     p1.m0 = m0;
     p1.t_in = a->first_sample;
