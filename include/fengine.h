@@ -94,8 +94,10 @@ typedef struct {
                                   with N2 <= 1024 (and N2 >= 512 / N1 for N1 > 8);
                                   built-in: max(8, N / 1024) */
     int32_t slab_spectra;      /* spectra per slab of the two-phase pipeline, a multiple
-                                  of 32; built-in: an intermediate of about 3 GiB (less
-                                  where the device has no room for it) */
+                                  of 32; built-in: as few slabs of equal size as keep the
+                                  intermediate of one within 3 GiB and 1/32 of the memory
+                                  that is free on the device when the plan is made (256 MiB
+                                  at least); a call of several slabs holds two */
     int64_t min_delay_samples; /* Dmin in [-2^30, 0]: the most negative coarse delay
                                   (Sec. 3.3 allows negative delays). The plan emits
                                   E = ceil(-Dmin / 2n) spectra later to make room. */
@@ -130,9 +132,10 @@ int32_t fengine_abi_version(void);
  * scaled so that sum w^2 = 1. out: host array of 2n*T floats. */
 fengine_status fengine_default_weights(int32_t n_channels, int32_t n_taps, float *out);
 
-/* The requantiser of one Gaussian-integer component that the kernels apply
- * (Sec. 2.1 step 6, Sec. 3.6): saturate to [-127, 127] and round half away
- * from zero, here evaluated on the host by the same steps. */
+/* The requantiser of one Gaussian-integer component (Sec. 2.1 step 6,
+ * Sec. 3.6): saturate to [-127, 127] and round half away from zero. This is
+ * the host's statement of the rule; the kernels apply it to four components
+ * at a time by steps of their own, with the same result for every value. */
 int32_t fengine_quantise(float x);
 
 /* Create a plan on the current CUDA device (use the plan only while that
@@ -282,12 +285,13 @@ fengine_status fengine_batch_destroy(fengine_batch_t batch);
 
 /* Process one chunk of each of n distinct plans as one call on cuda_stream:
  * every member computes exactly what fengine_process_chunk computes for it
- * (Sec. 2.1 steps 1-6). Members in the FP32 form are grouped: their small
- * per-call kernels run spread over the pool's streams, then their phase-1
- * and phase-2 work goes out as one grid per kernel instantiation (members
- * with the same taps and FFT split; up to 64 members per grid), slab by
- * slab, on cuda_stream. Members of the other forms run whole on the pool's
- * streams meanwhile, largest work first onto the least-loaded stream.
+ * (Sec. 2.1 steps 1-6). Members in the FP32 form are grouped: their prologues
+ * (delay tables, lost-data flags, history tails) are one grid on cuda_stream,
+ * then their phase-1 and phase-2 work goes out as one grid per kernel
+ * instantiation (members with the same taps and FFT split; up to 64 members
+ * per grid), slab by slab, each group on one of the pool's streams. Members
+ * of the other forms run whole on the pool's streams meanwhile, largest work
+ * first onto the least-loaded stream.
  * Everything forks from and joins back into cuda_stream (so the call can be
  * captured into a CUDA graph).
  * first_spectra (host, n entries, may be NULL) receives each member's first
@@ -528,9 +532,10 @@ fengine_status fengine_process_chunk_noalloc(const fengine_noalloc_args *args, c
 /* Per-stage device timing, a profiling aid. While enabled, every
  * fengine_process_chunk records CUDA events on its stream between its
  * kernels. fengine_stage_times waits for those events, writes the summed
- * milliseconds per stage to ms[0..4] = {delay table, phase 1 (FIR + first
- * FFT stage; in the FP32 form also the unpack), phase 2 (second FFT stage +
- * delay/gain + requantise + corner turn), history tail update, column unpack
+ * milliseconds per stage to ms[0..4] = {prologue (delay table, lost-data
+ * flags, history tail), phase 1 (FIR + first FFT stage; in the FP32 form also
+ * the unpack), phase 2 (second FFT stage + delay/gain + requantise + corner
+ * turn), 0 (the history tail is part of the prologue), column unpack
  * (tensor-core forms; 0 in the FP32 form)}, the number of timed calls to
  * *calls, and starts a new accumulation. ms holds 5 floats. Disabled by
  * default. */

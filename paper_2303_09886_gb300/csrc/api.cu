@@ -427,9 +427,10 @@ fengine_status fengine_plan_create(const fengine_config *cfg, fengine_plan_t *ou
     // stage takes the same time per spectrum from L2), so smaller slabs only
     // add launches and tails: 8192 channels, 4 antennas x 2 x 2^25 samples
     // take 0.89 ms as one slab and 1.02 ms as five of 256 MiB. Of the
-    // device's free memory a slab takes 1/32 at most, so that many plans fit
-    // side by side; the least is the 256 MiB slab. The plan's last allocation:
-    // it takes less where the device has no room for it next to the rest.
+    // device's free memory a slab takes 1/32 at most (a call of several slabs
+    // holds two), so that many plans fit side by side; the least is the 256
+    // MiB slab. The plan's last allocation: it takes less where the device has
+    // no room for it next to the rest.
     // intermediate element: FP32 (re, im), or FP16 (re, im) in the FP16 form
     pl->a_elem = pl->precision == FENGINE_TC_FP16 ? 4 : 8;
     const size_t per_spec = (size_t)ns * (pl->N1 / 2 + 1) * pl->N2 * pl->a_elem;

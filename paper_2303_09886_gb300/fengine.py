@@ -148,7 +148,7 @@ def _ptr(t):
 
 
 def quantise(x: float) -> int:
-    """The kernels' requantiser evaluated on the host (same source)."""
+    """The kernels' requantiser, as the host states the rule."""
     return int(load().fengine_quantise(float(x)))
 
 
