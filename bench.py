@@ -41,18 +41,18 @@ UNIT = "Gsample/s"
 # sources they were taken from (src = hash of the kernel's source files).
 KERNEL_SOURCES = {
     "k_phase1": ['k_phase1.cuh', 'k_phase1_t1.cu', 'k_phase1_t2.cu', 'k_phase1_t4.cu', 'k_phase1_t8.cu', 'k_phase1_t16.cu', 'k_phase1_t32.cu', 'fe_device.cuh', 'fe_internal.cuh'],
-    "k_phase2": ['k_phase2.cu', 'fe_device.cuh', 'fe_internal.cuh'],
-    "k_phase2w": ['k_phase2w.cu', 'fe_device.cuh', 'fe_internal.cuh'],
-    "k_phase1_tc": ['k_phase1_tc.cu', 'fe_device.cuh', 'fe_internal.cuh'],
+    "k_phase2": ['k_phase2.cu', 'k_phase2_tile.inc', 'fe_device.cuh', 'fe_internal.cuh'],
+    "k_phase2w": ['k_phase2w.cu', 'fe_waits.cuh', 'fe_device.cuh', 'fe_internal.cuh'],
+    "k_phase1_tc": ['k_phase1_tc.cu', 'fe_waits.cuh', 'fe_device.cuh', 'fe_internal.cuh'],
     "k_unpack_cols": ['k_phase1_tc.cu', 'fe_device.cuh', 'fe_internal.cuh'],
 }
 _CAPTURED = 33554432   # input samples of the captured launch
 NCU_TRAFFIC = {
-    "k_phase1<16,16,32,0>": {"bytes_per_sample": (44091392 + 90493184) / _CAPTURED, "src": "58685870f5a492cb"},
-    "k_phase2w": {"bytes_per_sample": (161295360 + 16910336) / _CAPTURED, "src": "d0c296192441a53f"},
-    "k_phase2w<half>": {"bytes_per_sample": (84109824 + 12113152) / _CAPTURED, "src": "d0c296192441a53f"},
-    "k_phase1_tc<2,16,1>": {"bytes_per_sample": (95922944 + 48432128) / _CAPTURED, "src": "581b89670166b1b5"},
-    "k_unpack_cols": {"bytes_per_sample": (42587904 + 19447296) / _CAPTURED, "src": "581b89670166b1b5"},
+    "k_phase1<16,16,32,0>": {"bytes_per_sample": (44080384 + 91264000) / _CAPTURED, "src": "cb8925b5bbc76e40"},
+    "k_phase2w": {"bytes_per_sample": (161309440 + 16882688) / _CAPTURED, "src": "9e3c9fa74e3474b4"},
+    "k_phase2w<half>": {"bytes_per_sample": (84172032 + 12058368) / _CAPTURED, "src": "9e3c9fa74e3474b4"},
+    "k_phase1_tc<2,16,1>": {"bytes_per_sample": (95700224 + 48500480) / _CAPTURED, "src": "cf113901b781ba95"},
+    "k_unpack_cols": {"bytes_per_sample": (42588672 + 19664128) / _CAPTURED, "src": "6ab999ae4fcc1a89"},
 }
 
 
