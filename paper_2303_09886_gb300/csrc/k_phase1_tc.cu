@@ -560,9 +560,10 @@ __global__ void __launch_bounds__(tc_threads(tc_one_cta(PH, R, T, PREC)), tc_one
             // -> 0.86 ms; 512 spectra of four of 8192, BF16, a step every 77, 0.473 ->
             // 0.394. Steps every 33 spectra and less in BF16 below 2048 channels are 2 - 3 %
             // the slower for it.)
-            constexpr int far = 1 << 20;   // (past every column)
-            const int dc = max(-far, min(far, ps.c0 - ps.c)), t_cg = cg * CW + dc;
-            if (!p.window_tap && t_cg >= 0 && t_cg + (PH - 1) % CW + N2 * ((PH - 1) / CW) < P) {   // none wraps
+            const int dc = ps.c0 - ps.c;
+            if (!p.window_tap && dc + cg * CW >= 0 && dc + (cg + 1) * CW <= N2) {
+                // every column sequence starts at row 8 (m0 + q0) - rb, 16-byte
+                // aligned, one bulk copy each (per plane)
                 if (ft == 0) {
                     constexpr uint32_t bytes = (uint32_t)(NPL * PH * XL * 2);
                     asm volatile("{\n\t.reg .b64 st;\n\tmbarrier.arrive.expect_tx.shared::cta.b64 st, [%0], %1;\n\t}"
@@ -582,13 +583,15 @@ __global__ void __launch_bounds__(tc_threads(tc_one_cta(PH, R, T, PREC)), tc_one
                 }
                 continue;
             }
+            constexpr int far = 1 << 20;   // (past every column)
+            const int t_cg = cg * CW + max(-far, min(far, dc));
             auto column = [&](int i) -> int { return t_cg + (i % CW) + N2 * (i / CW); };   // rises with i
             int w0 = 0, nw = 0;   // [w0, w0 + nw): the columns that wrap
             if (p.window_tap) {
                 nw = PH;
             } else if (t_cg < 0) {
                 while (nw < PH && column(nw) < 0) nw++;
-            } else {
+            } else if (column(PH - 1) >= P) {
                 while (nw < PH && column(PH - 1 - nw) >= P) nw++;
                 w0 = PH - nw;
             }
