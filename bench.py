@@ -50,9 +50,9 @@ _CAPTURED = 33554432   # input samples of the captured launch
 NCU_TRAFFIC = {
     "k_phase1<16,16,32,0>": {"bytes_per_sample": (44080384 + 91264000) / _CAPTURED, "src": "cb8925b5bbc76e40"},
     "k_phase2w": {"bytes_per_sample": (161309440 + 16882688) / _CAPTURED, "src": "9e3c9fa74e3474b4"},
-    "k_phase2w<half>": {"bytes_per_sample": (84172032 + 12058368) / _CAPTURED, "src": "9e3c9fa74e3474b4"},
-    "k_phase1_tc<2,16,1>": {"bytes_per_sample": (95700224 + 48500480) / _CAPTURED, "src": "cf113901b781ba95"},
-    "k_unpack_cols": {"bytes_per_sample": (42588672 + 19664128) / _CAPTURED, "src": "6ab999ae4fcc1a89"},
+    "k_phase2w<half>": {"bytes_per_sample": (84353792 + 12594176) / _CAPTURED, "src": "9e3c9fa74e3474b4"},
+    "k_phase1_tc<2,16,1>": {"bytes_per_sample": (95759360 + 48593408) / _CAPTURED, "src": "4e4af3e41b756ccf"},
+    "k_unpack_cols": {"bytes_per_sample": (42589952 + 20078848) / _CAPTURED, "src": "ed203907c6c72a9a"},
 }
 
 
